@@ -172,6 +172,11 @@ struct Level {
   float* dinv32 = nullptr;
   Csr P, R;
   float *pv32 = nullptr, *rv32 = nullptr;
+  // Q = P - D^-1 A P (l1-Jacobi levels with a coarser one): CSR and length-sorted SELL-32
+  Csr Q;
+  float* qv32 = nullptr;
+  Sell qsell;
+  unsigned char* qperm = nullptr;
   Csr AT;
   float* atv32 = nullptr;
   Sell sellT;
@@ -309,9 +314,10 @@ static Csr transpose(Arena& a, const Csr& X, cudaStream_t s, Scratch* keep = nul
 }
 
 // SELL-32 copy of A in the V-cycle's precision only (FP32 values when mixed,
-// else FP64); with dinv given, also A D^-1 in the same layout (vpre).
+// else FP64); with dinv given, also A D^-1 in the same layout (vpre); the
+// values themselves only with `values` (levels with Q never read them).
 static Sell build_sell(Arena& a, const Csr& A, bool mixed, cudaStream_t s, const int* selfmap = nullptr,
-                       const double* dinv = nullptr) {
+                       const double* dinv = nullptr, bool values = true) {
   Scratch sc(s);
   Sell S;
   S.n = A.n;
@@ -323,15 +329,50 @@ static Sell build_sell(Arena& a, const Csr& A, bool mixed, cudaStream_t s, const
   S.nstored = read_int(S.sptr + S.nslices, s);
   S.ci = a.alloc<int>(S.nstored);
   if (mixed) {
-    S.v32 = a.alloc<float>(S.nstored);
+    if (values) S.v32 = a.alloc<float>(S.nstored);
     if (dinv) S.vpre32 = a.alloc<float>(S.nstored);
     launch_sell_fill(A.n, A.rp, A.ci, A.v, dinv, S.sptr, S.ci, S.v32, S.vpre32, s, selfmap);
   } else {
-    S.v = a.alloc<double>(S.nstored);
+    if (values) S.v = a.alloc<double>(S.nstored);
     if (dinv) S.vpre = a.alloc<double>(S.nstored);
     launch_sell_fill(A.n, A.rp, A.ci, A.v, dinv, S.sptr, S.ci, S.v, S.vpre, s, selfmap);
   }
   return S;
+}
+
+// The level's smoother diagonal D^-1 = 1 / sum_j |a_ij|
+static void build_dinv(Arena& a, Level& lv, bool mixed, cudaStream_t s) {
+  if (lv.dinv) return;
+  lv.dinv = a.alloc<double>(lv.A.n);
+  if (mixed) lv.dinv32 = a.alloc<float>(lv.A.n);
+  launch_l1_dinv(lv.A.n, lv.A.rp, lv.A.v, lv.dinv, s, lv.dinv32);
+}
+
+// Q = P - D^-1 A P of a level from its A P (arena arrays, turned into Q in place)
+static void build_q(Arena& a, Level& lv, const Csr& AP, bool mixed, cudaStream_t s) {
+  Scratch sc(s);
+  const int n = AP.n, nwin = (n + kQWin - 1) / kQWin;
+  Sell& S = lv.qsell;
+  lv.Q = AP;
+  S.n = n;
+  S.nslices = nwin * (kQWin / 32);
+  lv.qperm = a.alloc<unsigned char>((size_t)nwin * kQWin);
+  int* w = sc.alloc<int>(S.nslices);
+  launch_q_order(n, AP.rp, lv.qperm, w, s);
+  S.sptr = a.alloc<int>(S.nslices + 1);
+  exclusive_scan(w, S.sptr, S.nslices, s);
+  S.nstored = read_int(S.sptr + S.nslices, s);
+  S.ci = a.alloc<int>(S.nstored);
+  if (mixed) {
+    lv.qv32 = a.alloc<float>(AP.nnz);
+    S.v32 = a.alloc<float>(S.nstored);
+    launch_q_fill<float>(n, AP.rp, AP.ci, AP.v, lv.qv32, lv.P.rp, lv.P.ci, lv.P.v, lv.dinv, lv.qperm, S.sptr, S.ci,
+                         S.v32, s);
+  } else {
+    S.v = a.alloc<double>(S.nstored);
+    launch_q_fill<double>(n, AP.rp, AP.ci, AP.v, nullptr, lv.P.rp, lv.P.ci, lv.P.v, lv.dinv, lv.qperm, S.sptr, S.ci,
+                          S.v, s);
+  }
 }
 
 static float* cast32(Arena& a, const double* x, int n, cudaStream_t s) {
@@ -553,12 +594,18 @@ static void build_hierarchy(SetupCtx& sc, Hier& h, const Csr& A0) {
     lv.R = transpose(ar, P, s);
     pt_tr.stop();
     PhaseTimer pt_ap(sc.clk, SP_AP);
+    const bool with_q = lv.nk == 0;  // A P stays as Q on l1-Jacobi levels
     Scratch apk(s, ar.pool);
-    Csr AP = spgemm(ar, lv.A, P, s, &apk);
+    Csr AP = spgemm(ar, lv.A, P, s, with_q ? nullptr : &apk);
     pt_ap.stop();
     PhaseTimer pt_rap(sc.clk, SP_RAP);
     Csr Ac = spgemm(ar, lv.R, AP, s);
     pt_rap.stop();
+    if (with_q) {
+      PhaseTimer pt_q(sc.clk, SP_FINALIZE);
+      build_dinv(ar, lv, sc.mixed, s);
+      build_q(ar, lv, AP, sc.mixed, s);
+    }
     h.L.emplace_back();
     h.L.back().A = Ac;
   }
@@ -567,9 +614,7 @@ static void build_hierarchy(SetupCtx& sc, Hier& h, const Csr& A0) {
   for (int l = 0; l < h.nlev(); ++l) {
     Level& lv = h.L[l];
     int n = lv.A.n;
-    lv.dinv = ar.alloc<double>(n);
-    if (sc.mixed) lv.dinv32 = ar.alloc<float>(n);
-    launch_l1_dinv(n, lv.A.rp, lv.A.v, lv.dinv, s, lv.dinv32);
+    build_dinv(ar, lv, sc.mixed, s);
     if (lv.nk > 0) {
       lv.gdinv = ar.alloc<double>(n);
       launch_diag_inv(n, lv.A.rp, lv.A.ci, lv.A.v, lv.gdinv, s);
@@ -594,7 +639,7 @@ static void build_hierarchy(SetupCtx& sc, Hier& h, const Csr& A0) {
     // value (or the FP64 product a_ij d_j) rounded once.
     const bool jac = lv.nk == 0;
     const double* pre = jac ? lv.dinv : nullptr;
-    lv.sell = build_sell(ar, lv.A, sc.mixed, s, nullptr, pre);
+    lv.sell = build_sell(ar, lv.A, sc.mixed, s, nullptr, pre, lv.qperm == nullptr);
     if (sc.mixed) {
       lv.v32 = ar.alloc<float>(lv.A.nnz);
       if (jac) lv.vpre32 = ar.alloc<float>(lv.A.nnz);
@@ -680,6 +725,7 @@ struct VBatch {
   double bytes_total = 0;
   // fused coarse-level kernel: levels >= tail_level of every subsystem in one
   // cluster launch (tail_level >= depth: not used)
+    bool q = false;  // the way up is POSTQ (every subsystem has Q), its layout fmtP
   int tail_level = 1 << 20;
   int tail_cs = 8;
   TailSub<T>* d_tail = nullptr;
@@ -751,6 +797,13 @@ static double sp_bytes(long long nnz, long long rows, int sv) { return (double)n
 
 template <typename T>
 static void build_plan(Arena& ar, VBatch<T>& vb, bool trans, cudaStream_t s) {
+    d.qrp = lv.Q.rp;
+    d.qci = lv.Q.ci;
+    d.qv = pick<T>(lv.Q.v, lv.qv32);
+    d.qsptr = lv.qsell.sptr;
+    d.qsci = lv.qsell.ci;
+    d.qsv = pick<T>(lv.qsell.v, lv.qsell.v32);
+    d.qperm = lv.qperm;
   auto& plan = trans ? vb.planT : vb.plan;
   vb.depth = 0;
   for (Hier* h : vb.hs) vb.depth = std::max(vb.depth, h->nlev());
@@ -791,15 +844,18 @@ static void build_plan(Arena& ar, VBatch<T>& vb, bool trans, cudaStream_t s) {
                           sp_bytes(nnz, n, sv) + 3.0 * sv * n;
           lp.bytes_post += sp_bytes(nnz, n, sv) + (4.0 + 4.0 * sv) * n;
         } else {
-          lp.bytes_pre += sp_bytes(nnz, n, sv) + 4.0 * sv * n;
-          lp.bytes_post += sp_bytes(nnz, n, sv) + 4.0 * sv * n;
-          if (sv == 8) {  // k_pre: a multiply-add per nonzero, xt = D^-1 b, r = b - s; k_post likewise
+          // with Q the way up reads it, xc, b, r and D^-1 and writes x; PRE then forms no xt
+          lp.q = d.qperm != nullptr;
+          lp.bytes_pre += sp_bytes(nnz, n, sv) + (lp.q ? 2.0 : 4.0) * sv * n;
+          lp.bytes_post += lp.q ? sp_bytes(lv.Q.nnz, n, sv) + n + (double)sv * (lv.nc + 4.0 * n)
+                                : sp_bytes(nnz, n, sv) + 4.0 * sv * n;
+          if (sv == 8) {  // the method's count: a multiply-add per nonzero of A and two per row, before and after
             lp.fp64_pre += (double)nnz + 2.0 * n;
             lp.fp64_post += (double)nnz + 2.0 * n;
           }
         }
         lp.bytes_restrict += sp_bytes(lv.R.nnz, lv.nc, sv) + (double)sv * (n + lv.nc);
-        lp.bytes_prolong += sp_bytes(lv.P.nnz, n, sv) + (double)sv * (lv.nc + 2 * n);
+        if (!lp.q) lp.bytes_prolong += sp_bytes(lv.P.nnz, n, sv) + (double)sv * (lv.nc + 2 * n);
       } else if (h->coarse_lu) {
         clu.push_back(d);
         lp.maxcn = std::max(lp.maxcn, h->cn);
@@ -884,10 +940,13 @@ static void run_vbatch(VBatch<T>& vb, bool trans, cudaStream_t s, Profiler& prof
   for (int l = std::min(vb.depth - 2, ltop - 1); l >= 0; --l) {
     auto& lp = plan[l];
     if (!lp.ndown) continue;
-    prof.next_detail = 16 + 4 * l + 2;
-    int id = prof.begin(s, 1);
-    launch_phase<T>(PH_PROLONG, lp.fmtA, lp.fmtP, lp.d_down, lp.ndown, lp.maxn, s);
-    prof.end(id, 1, lp.bytes_prolong, s);
+    int id;
+    if (!lp.q) {
+      prof.next_detail = 16 + 4 * l + 2;
+      id = prof.begin(s, 1);
+      launch_phase<T>(PH_PROLONG, lp.fmtA, lp.fmtP, lp.d_down, lp.ndown, lp.maxn, s);
+      prof.end(id, 1, lp.bytes_prolong, s);
+    }
     prof.next_detail = 16 + 4 * l + 3;
     id = prof.begin(s, l == 0 ? 0 : 1);
     if (lp.gs) run_gs_up<T>(lp, s);
@@ -904,6 +963,7 @@ static void build_tail(Arena& ar, VBatch<T>& vb, int Lt, bool keepT, cudaStream_
   vb.ntail = 0;
   vb.tail_bytes = 0;
   if (Lt >= vb.depth) return;
+    else if (lp.q) launch_phase<T>(PH_POSTQ, lp.fmtA, lp.fmtP, lp.d_down, lp.ndown, lp.maxn, s);
   for (int pass = 0; pass < (keepT ? 2 : 1); ++pass) {
     bool trans = pass == 1;
     std::vector<TailSub<T>> subs;
@@ -1147,6 +1207,7 @@ struct mgd_ctx {
   std::string err;
   mgd::Pool pool;
   mgd::Arena ar;
+  const int candQ[] = {FMT_CSR1, FMT_CSR2, FMT_CSR4, FMT_CSR8};  // CSR1: the length-sorted SELL-32 (same sums)
   bool ready = false;
   int kind = 0, G = 0, N = 0, n = 0, nnz = 0;
   mgd::Csr A;      // monolithic operator (FP64)
@@ -1184,7 +1245,16 @@ struct mgd_ctx {
 
 namespace mgd {
 
+    for (int f : candQ) {
+      if (!lp.q) break;
+      float ms = time_it([&] { launch_phase<T>(PH_POSTQ, lp.fmtA, f, lp.d_down, lp.ndown, lp.maxn, s); });
+      if (ms < best) {
+        best = ms;
+        lp.fmtP = f;
+      }
+    }
 static bool mixed(const mgd_ctx* c) { return c->o.precision == 1; }
+      if (lp.q) break;
 
 static PRef ABS(double* p) { return PRef{0, 0, p}; }
 static PRef VIN(long long off) { return PRef{1, off, nullptr}; }

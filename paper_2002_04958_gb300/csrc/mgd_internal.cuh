@@ -319,6 +319,16 @@ struct LDesc {
   const int* rrp;
   const int* rci;
   const T* rv;
+  // Q = P - D^-1 A P, the correction and the post-smoothing of an l1-Jacobi
+  // level as one operator (nullptr: not built): CSR, and SELL-32 with the rows
+  // of each 256-row window sorted by length (qperm: sorted place -> row)
+  const int* qrp;
+  const int* qci;
+  const T* qv;
+  const int* qsptr;
+  const int* qsci;
+  const T* qsv;
+  const unsigned char* qperm;
   // vectors
   T* b;   // right-hand side of this level
   T* x;   // output of this level's cycle
@@ -524,9 +534,17 @@ void launch_grad_vals(int n, const int* rp, const int* ci, const double* x, cons
 void launch_offsets64(const int* cnt, long long* off, int n, cudaStream_t s);
 
 // ------------------------------------------------------------------ solve launchers (solve_kernels.cu)
-enum Phase { PH_PRE = 0, PH_RESTRICT = 1, PH_PROLONG = 2, PH_POST = 3, PH_COARSE = 4, PH_JAC1 = 5 };
+enum Phase { PH_PRE = 0, PH_RESTRICT = 1, PH_PROLONG = 2, PH_POST = 3, PH_COARSE = 4, PH_JAC1 = 5, PH_POSTQ = 6 };
 
 template <typename T>
+// Q = P - D^-1 A P (see k_q_fill): the window order and the slice widths, then
+// the values (q holds A P on entry, Q on return; q32: its FP32 copy, or nullptr)
+constexpr int kQWin = 256;  // rows per window
+void launch_q_order(int n, const int* rp, unsigned char* perm, int* widths, cudaStream_t s);
+template <typename T>
+void launch_q_fill(int n, const int* rp, const int* ci, double* q, float* q32, const int* prp, const int* pci,
+                   const double* pv, const double* dinv, const unsigned char* perm, const int* sptr, int* sci, T* sv,
+                   cudaStream_t s);
 void launch_phase(int phase, int fmtA, int tprRP, const LDesc<T>* d_descs, int ndesc, int maxrows,
                   cudaStream_t s);
 // Gauss-Seidel smoothing phases (levels with nk > 0)

@@ -1799,11 +1799,11 @@ __global__ void k_sell_fill(int n, const int* rp, const int* ci, const double* v
       int c = ci[b + j];
       double a = v[b + j];
       sci[idx] = c;
-      sv[idx] = (T)a;
+      if (sv) sv[idx] = (T)a;
       if (svpre) svpre[idx] = (T)__dmul_rn(a, d[c]);
     } else {
       sci[idx] = self;
-      sv[idx] = T(0);
+      if (sv) sv[idx] = T(0);
       if (svpre) svpre[idx] = T(0);
     }
   }
@@ -1827,6 +1827,84 @@ void launch_sell_fill(int n, const int* rp, const int* ci, const double* v, cons
                       int* sci, float* sv, float* svpre, cudaStream_t s, const int* selfmap) {
   sell_fill<float>(n, rp, ci, v, d, sptr, sci, sv, svpre, s, selfmap);
 }
+
+// ------------------------------------------------------------------ Q = P - D^-1 A P
+// One block per 256-row window: each row's place in the window's order by
+// length (longest first, equal lengths by index; rows past n last), and the
+// width of each of its eight 32-row slices, the length of its first row.
+__global__ void __launch_bounds__(kQWin) k_q_order(int n, const int* rp, unsigned char* perm, int* widths) {
+  __shared__ int s_len[kQWin];
+  const int t = threadIdx.x, r = blockIdx.x * kQWin + t;
+  const int len = r < n ? rp[r + 1] - rp[r] : -1;
+  s_len[t] = len;
+  __syncthreads();
+  int place = 0;
+  for (int j = 0; j < kQWin; ++j) {
+    const int o = s_len[j];
+    place += o > len || (o == len && j < t);
+  }
+  perm[(size_t)blockIdx.x * kQWin + place] = (unsigned char)t;
+  if ((place & 31) == 0) widths[blockIdx.x * (kQWin / 32) + (place >> 5)] = 32 * max(len, 0);
+}
+
+void launch_q_order(int n, const int* rp, unsigned char* perm, int* widths, cudaStream_t s) {
+  k_q_order<<<cdiv(n, kQWin), kQWin, 0, s>>>(n, rp, perm, widths);
+  MGD_LAUNCH_CHECK();
+}
+
+// The values of Q on the pattern of A P (its row i holds P's row i: a_ii is
+// stored): q_ic = p_ic - d_i (A P)_ic, in place in the CSR values and copied
+// to the sorted SELL-32 layout.  A thread per sorted place merges its rows of
+// A P and P, both in increasing column order.  Padding is a zero at the row's
+// first column.
+template <typename T>
+__global__ void __launch_bounds__(kQWin) k_q_fill(int n, const int* rp, const int* ci, double* q, float* q32,
+                                                  const int* prp, const int* pci, const double* pv,
+                                                  const double* dinv, const unsigned char* perm, const int* sptr,
+                                                  int* sci, T* sv) {
+  const int place = blockIdx.x * kQWin + threadIdx.x;
+  const int r = blockIdx.x * kQWin + perm[place];
+  const int base = sptr[place >> 5], width = (sptr[(place >> 5) + 1] - base) >> 5;
+  int b = 0, e = 0, pp = 0, pe = 0;
+  double d = 0.0;
+  if (r < n) {
+    b = rp[r];
+    e = rp[r + 1];
+    pp = prp[r];
+    pe = prp[r + 1];
+    d = dinv[r];
+  }
+  const int first = e > b ? ci[b] : 0;
+  for (int j = 0; j < width; ++j) {
+    const size_t idx = (size_t)base + 32 * (size_t)j + (place & 31);
+    int c = first;
+    T out = T(0);
+    if (b + j < e) {
+      c = ci[b + j];
+      double v = -__dmul_rn(d, q[b + j]);
+      if (pp < pe && pci[pp] == c) v = __dadd_rn(v, pv[pp++]);
+      q[b + j] = v;
+      if (q32) q32[b + j] = (float)v;
+      out = (T)v;
+    }
+    sci[idx] = c;
+    sv[idx] = out;
+  }
+}
+
+template <typename T>
+void launch_q_fill(int n, const int* rp, const int* ci, double* q, float* q32, const int* prp, const int* pci,
+                   const double* pv, const double* dinv, const unsigned char* perm, const int* sptr, int* sci, T* sv,
+                   cudaStream_t s) {
+  k_q_fill<T><<<cdiv(n, kQWin), kQWin, 0, s>>>(n, rp, ci, q, q32, prp, pci, pv, dinv, perm, sptr, sci, sv);
+  MGD_LAUNCH_CHECK();
+}
+template void launch_q_fill<double>(int, const int*, const int*, double*, float*, const int*, const int*,
+                                    const double*, const double*, const unsigned char*, const int*, int*, double*,
+                                    cudaStream_t);
+template void launch_q_fill<float>(int, const int*, const int*, double*, float*, const int*, const int*,
+                                   const double*, const double*, const unsigned char*, const int*, int*, float*,
+                                   cudaStream_t);
 
 // ------------------------------------------------------------------ column scaling A D^-1
 // out = A D^-1 values (the FP64 product, rounded to T); vout, when given, the

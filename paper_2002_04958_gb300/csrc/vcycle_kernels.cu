@@ -30,7 +30,8 @@ constexpr int kVThreads = MGD_VTHREADS;
 constexpr int kPre = MGD_KPRE;  // entries per lane loaded before the wait
 
 // PRE: xt = D^-1 b (zero initial guess), r = b - A xt = b - (A D^-1) b, using
-// the column-scaled copy of A so that each nonzero costs one multiply-add
+// the column-scaled copy of A so that each nonzero costs one multiply-add.
+// Levels with Q (POSTQ below) need no xt: it is not formed there.
 template <typename T, int FMT>
 __global__ void __launch_bounds__(kVThreads) k_pre(const LDesc<T>* __restrict__ descs) {
   MGD_PDL_TRIGGER();
@@ -51,7 +52,7 @@ __global__ void __launch_bounds__(kVThreads) k_pre(const LDesc<T>* __restrict__ 
   T s = row_finish<T, FMT, kPre>(R, valid, d->ci, d->vpre, d->sci, d->svpre, xf);
   if (valid && lane == 0) {
     T bi = b[row];
-    d->xt[row] = di * bi;
+    if (!d->qperm) d->xt[row] = di * bi;
     d->r[row] = bi - s;
   }
 }
@@ -106,7 +107,7 @@ __global__ void __launch_bounds__(kVThreads) k_pre_sk(const LDesc<T>* __restrict
     T s = row_finish<T, FMT_SELL, kPre>(R[q], r < n, nullptr, nullptr, d->sci, d->svpre, xf);
     if (r < n) {
       T bi = b[r];
-      d->xt[r] = di[q] * bi;
+      if (!d->qperm) d->xt[r] = di[q] * bi;
       d->r[r] = bi - s;
     }
   }
@@ -137,6 +138,60 @@ __global__ void __launch_bounds__(kVThreads) k_post_sk(const LDesc<T>* __restric
     T s = row_finish<T, FMT_SELL, kPre>(R[q], r < n, nullptr, nullptr, d->sci, d->sv, xf);
     if (r < n) d->x[r] = d->xt[r] + di[q] * (d->b[r] - s);
   }
+}
+
+// POSTQ: prolongation and post-smoothing as one product.  With xt = D^-1 b and
+// r = b - A xt from PRE, the correction xt + P xc and the sweep after it are
+//   x = xt + P xc + D^-1 (b - A (xt + P xc)) = D^-1 (b + r) + (P - D^-1 A P) xc,
+// and Q = P - D^-1 A P has the pattern of A P, which the setup forms anyway:
+// 6.5 entries a row on a 7-point level 0 (A 6.9), 8.8 on level 1 (A 15.9).  So
+// neither A nor P is read on the way up, xt is neither written nor updated,
+// and a level takes three launches instead of four.  Bound by HBM and by the
+// FP64 pipe alike (one multiply-add per 12 bytes), so padding costs twice:
+// rows of Q differ in length (SELL-32 would pad 6.5 to 11.9 entries), and the
+// rows of a 256-row window are sorted by length, one window per block; the
+// sums return to natural order through shared memory, so that every vector
+// access stays coalesced.  A row is summed in CSR order.  Measured on the 21
+// subsystems of 884,736 rows (FP64): level 0 668 -> 499 us (262 prolongation +
+// 406 post-smoothing; 4.5 TB/s), level 1 346 -> 183 us, an apply 2.48 -> 2.05 ms.
+template <typename T>
+__global__ void __launch_bounds__(kQWin) k_postq(const LDesc<T>* __restrict__ descs) {
+  __shared__ T s_sum[kQWin];
+  MGD_PDL_TRIGGER();
+  const LDesc<T>* d = descs + blockIdx.y;
+  const int n = d->n, t = threadIdx.x;
+  const int row = blockIdx.x * kQWin + t;  // this thread's row of the vectors, and its sorted place
+  if ((int)blockIdx.x * kQWin >= n) return;
+  const int mine = d->qperm[row];          // (the window's last places hold the rows past n)
+  RowPre<T, kPre> R;
+  row_load<T, FMT_SELL, kPre>(R, row, 0, true, nullptr, nullptr, nullptr, d->qsptr, d->qsci, d->qsv);
+  const T di = row < n ? d->dinv[row] : T(0);
+  MGD_PDL_WAIT();
+  MGD_SKIP_INACTIVE(d);
+  s_sum[mine] = row_finish<T, FMT_SELL, kPre>(R, true, nullptr, nullptr, d->qsci, d->qsv, XPlain<T>{d->xc});
+  __syncthreads();
+  if (row < n) d->x[row] = di * (d->b[row] + d->r[row]) + s_sum[t];
+}
+
+// the same from CSR with TPR threads per row (short levels, where a row's
+// entries taken one by one would be the whole kernel's time)
+template <typename T, int FMT>
+__global__ void __launch_bounds__(kVThreads) k_postq_csr(const LDesc<T>* __restrict__ descs) {
+  MGD_PDL_TRIGGER();
+  const LDesc<T>* d = descs + blockIdx.y;
+  constexpr int TPR = FmtTraits<FMT>::tpr;
+  int g = blockIdx.x * blockDim.x + threadIdx.x;
+  int row = g / TPR, lane = g % TPR;
+  int n = d->n;
+  if (((g & ~31) / TPR) >= n) return;
+  bool valid = row < n;
+  RowPre<T, kPre> R;
+  row_load<T, FMT, kPre>(R, row, lane, valid, d->qrp, d->qci, d->qv, nullptr, nullptr, nullptr);
+  T di = valid && lane == 0 ? d->dinv[row] : T(0);
+  MGD_PDL_WAIT();
+  MGD_SKIP_INACTIVE(d);
+  T s = row_finish<T, FMT, kPre>(R, valid, d->qci, d->qv, nullptr, nullptr, XPlain<T>{d->xc});
+  if (valid && lane == 0) d->x[row] = di * (d->b[row] + d->r[row]) + s;
 }
 
 // RESTRICT: bc = R r ; PROLONG: xt += P xc  (CSR, TPR threads per row)
@@ -379,6 +434,16 @@ template void launch_phase<float>(int, int, int, const LDesc<float>*, int, int, 
 // every point reads only values of other sweeps.  x is the same buffer as xt
 // on these levels.
 template <typename T>
+    case PH_POSTQ:
+      switch (fmtRP) {
+        case FMT_CSR2: launch_k(k_postq_csr<T, FMT_CSR2>, dim3(cdiv(2LL * maxrows, kVThreads), ndesc), dim3(kVThreads), 0, s, d_descs); break;
+        case FMT_CSR4: launch_k(k_postq_csr<T, FMT_CSR4>, dim3(cdiv(4LL * maxrows, kVThreads), ndesc), dim3(kVThreads), 0, s, d_descs); break;
+        case FMT_CSR8: launch_k(k_postq_csr<T, FMT_CSR8>, dim3(cdiv(8LL * maxrows, kVThreads), ndesc), dim3(kVThreads), 0, s, d_descs); break;
+        case FMT_CSR16: launch_k(k_postq_csr<T, FMT_CSR16>, dim3(cdiv(16LL * maxrows, kVThreads), ndesc), dim3(kVThreads), 0, s, d_descs); break;
+        case FMT_CSR32: launch_k(k_postq_csr<T, FMT_CSR32>, dim3(cdiv(32LL * maxrows, kVThreads), ndesc), dim3(kVThreads), 0, s, d_descs); break;
+        default: launch_k(k_postq<T>, dim3(cdiv(maxrows, kQWin), ndesc), dim3(kQWin), 0, s, d_descs); break;
+      }
+      break;
 __global__ void k_gs_first(const LDesc<T>* __restrict__ descs) {
   MGD_PDL_ENTRY();
   const LDesc<T>* d = descs + blockIdx.y;
