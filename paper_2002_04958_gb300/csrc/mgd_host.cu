@@ -717,6 +717,7 @@ struct VBatch {
     double fp64_pre = 0, fp64_post = 0, fp64_cj = 0;
     // Gauss-Seidel levels: sweep steps and, per step, the largest class over the subsystems
     bool gs = false;
+    bool q = false;  // the way up is POSTQ (every subsystem has Q), its layout fmtP
     int nkmax = 0, fmtGS = FMT_CSR4;  // sweep layout; SELL only where the sweep-ordered copy exists
     bool gs_sell = false;
     std::vector<int> seg_pre, seg_post;
@@ -725,7 +726,6 @@ struct VBatch {
   double bytes_total = 0;
   // fused coarse-level kernel: levels >= tail_level of every subsystem in one
   // cluster launch (tail_level >= depth: not used)
-    bool q = false;  // the way up is POSTQ (every subsystem has Q), its layout fmtP
   int tail_level = 1 << 20;
   int tail_cs = 8;
   TailSub<T>* d_tail = nullptr;
@@ -786,6 +786,13 @@ static LDesc<T> make_desc(Hier& h, int l, bool trans) {
   d.koff = lv.koff;
   d.gdinv = pick<T>(lv.gdinv, lv.gdinv32);
   if (!trans) {
+    d.qrp = lv.Q.rp;
+    d.qci = lv.Q.ci;
+    d.qv = pick<T>(lv.Q.v, lv.qv32);
+    d.qsptr = lv.qsell.sptr;
+    d.qsci = lv.qsell.ci;
+    d.qsv = pick<T>(lv.qsell.v, lv.qsell.v32);
+    d.qperm = lv.qperm;
     d.gsptr = lv.gsell.sptr;
     d.gsci = lv.gsell.ci;
     d.gsv = pick<T>(lv.gsell.v, lv.gsell.v32);
@@ -797,13 +804,6 @@ static double sp_bytes(long long nnz, long long rows, int sv) { return (double)n
 
 template <typename T>
 static void build_plan(Arena& ar, VBatch<T>& vb, bool trans, cudaStream_t s) {
-    d.qrp = lv.Q.rp;
-    d.qci = lv.Q.ci;
-    d.qv = pick<T>(lv.Q.v, lv.qv32);
-    d.qsptr = lv.qsell.sptr;
-    d.qsci = lv.qsell.ci;
-    d.qsv = pick<T>(lv.qsell.v, lv.qsell.v32);
-    d.qperm = lv.qperm;
   auto& plan = trans ? vb.planT : vb.plan;
   vb.depth = 0;
   for (Hier* h : vb.hs) vb.depth = std::max(vb.depth, h->nlev());
@@ -950,6 +950,7 @@ static void run_vbatch(VBatch<T>& vb, bool trans, cudaStream_t s, Profiler& prof
     prof.next_detail = 16 + 4 * l + 3;
     id = prof.begin(s, l == 0 ? 0 : 1);
     if (lp.gs) run_gs_up<T>(lp, s);
+    else if (lp.q) launch_phase<T>(PH_POSTQ, lp.fmtA, lp.fmtP, lp.d_down, lp.ndown, lp.maxn, s);
     else launch_phase<T>(PH_POST, lp.fmtA, lp.fmtP, lp.d_down, lp.ndown, lp.maxn, s);
     prof.end(id, l == 0 ? 0 : 1, lp.bytes_post, s, lp.gs ? 0.0 : lp.fp64_post);
   }
@@ -963,7 +964,6 @@ static void build_tail(Arena& ar, VBatch<T>& vb, int Lt, bool keepT, cudaStream_
   vb.ntail = 0;
   vb.tail_bytes = 0;
   if (Lt >= vb.depth) return;
-    else if (lp.q) launch_phase<T>(PH_POSTQ, lp.fmtA, lp.fmtP, lp.d_down, lp.ndown, lp.maxn, s);
   for (int pass = 0; pass < (keepT ? 2 : 1); ++pass) {
     bool trans = pass == 1;
     std::vector<TailSub<T>> subs;
@@ -1092,6 +1092,7 @@ static void autotune(VBatch<T>& vb, bool trans, cudaStream_t s) {
   };
   const int candA[] = {FMT_SELL, FMT_SELL2, FMT_SELL4, FMT_CSR1, FMT_CSR2, FMT_CSR4, FMT_CSR8};
   const int candRP[] = {FMT_CSR1, FMT_CSR1X2, FMT_CSR1X4, FMT_CSR2, FMT_CSR4, FMT_CSR8};
+  const int candQ[] = {FMT_CSR1, FMT_CSR2, FMT_CSR4, FMT_CSR8};  // CSR1: the length-sorted SELL-32 (same sums)
   for (int l = 0; l < vb.depth; ++l) {
     auto& lp = plan[l];
     if (!lp.ndown) continue;
@@ -1129,7 +1130,16 @@ static void autotune(VBatch<T>& vb, bool trans, cudaStream_t s) {
       }
     }
     best = 1e30f;
+    for (int f : candQ) {
+      if (!lp.q) break;
+      float ms = time_it([&] { launch_phase<T>(PH_POSTQ, lp.fmtA, f, lp.d_down, lp.ndown, lp.maxn, s); });
+      if (ms < best) {
+        best = ms;
+        lp.fmtP = f;
+      }
+    }
     for (int f : candRP) {
+      if (lp.q) break;
       float ms = time_it([&] { launch_phase<T>(PH_PROLONG, lp.fmtA, f, lp.d_down, lp.ndown, lp.maxn, s); });
       if (ms < best) {
         best = ms;
@@ -1207,7 +1217,6 @@ struct mgd_ctx {
   std::string err;
   mgd::Pool pool;
   mgd::Arena ar;
-  const int candQ[] = {FMT_CSR1, FMT_CSR2, FMT_CSR4, FMT_CSR8};  // CSR1: the length-sorted SELL-32 (same sums)
   bool ready = false;
   int kind = 0, G = 0, N = 0, n = 0, nnz = 0;
   mgd::Csr A;      // monolithic operator (FP64)
@@ -1245,16 +1254,7 @@ struct mgd_ctx {
 
 namespace mgd {
 
-    for (int f : candQ) {
-      if (!lp.q) break;
-      float ms = time_it([&] { launch_phase<T>(PH_POSTQ, lp.fmtA, f, lp.d_down, lp.ndown, lp.maxn, s); });
-      if (ms < best) {
-        best = ms;
-        lp.fmtP = f;
-      }
-    }
 static bool mixed(const mgd_ctx* c) { return c->o.precision == 1; }
-      if (lp.q) break;
 
 static PRef ABS(double* p) { return PRef{0, 0, p}; }
 static PRef VIN(long long off) { return PRef{1, off, nullptr}; }

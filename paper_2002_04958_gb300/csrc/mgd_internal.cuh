@@ -525,6 +525,14 @@ void launch_sell_fill(int n, const int* rp, const int* ci, const double* v, cons
                       int* sci, double* sv, double* svpre, cudaStream_t s, const int* selfmap = nullptr);
 void launch_sell_fill(int n, const int* rp, const int* ci, const double* v, const double* d, const int* sptr,
                       int* sci, float* sv, float* svpre, cudaStream_t s, const int* selfmap = nullptr);
+// Q = P - D^-1 A P (see k_q_fill): the window order and the slice widths, then
+// the values (q holds A P on entry, Q on return; q32: its FP32 copy, or nullptr)
+constexpr int kQWin = 256;  // rows per window
+void launch_q_order(int n, const int* rp, unsigned char* perm, int* widths, cudaStream_t s);
+template <typename T>
+void launch_q_fill(int n, const int* rp, const int* ci, double* q, float* q32, const int* prp, const int* pci,
+                   const double* pv, const double* dinv, const unsigned char* perm, const int* sptr, int* sci, T* sv,
+                   cudaStream_t s);
 void launch_colscale(long long nnz, const int* ci, const double* v, const double* d, double* out, cudaStream_t s);
 // FP32 values (vout) and FP32 A D^-1 (out, when d is given) of FP64 CSR values, one pass
 void launch_colscale_f32(long long nnz, const int* ci, const double* v, const double* d, float* vout, float* out,
@@ -537,14 +545,6 @@ void launch_offsets64(const int* cnt, long long* off, int n, cudaStream_t s);
 enum Phase { PH_PRE = 0, PH_RESTRICT = 1, PH_PROLONG = 2, PH_POST = 3, PH_COARSE = 4, PH_JAC1 = 5, PH_POSTQ = 6 };
 
 template <typename T>
-// Q = P - D^-1 A P (see k_q_fill): the window order and the slice widths, then
-// the values (q holds A P on entry, Q on return; q32: its FP32 copy, or nullptr)
-constexpr int kQWin = 256;  // rows per window
-void launch_q_order(int n, const int* rp, unsigned char* perm, int* widths, cudaStream_t s);
-template <typename T>
-void launch_q_fill(int n, const int* rp, const int* ci, double* q, float* q32, const int* prp, const int* pci,
-                   const double* pv, const double* dinv, const unsigned char* perm, const int* sptr, int* sci, T* sv,
-                   cudaStream_t s);
 void launch_phase(int phase, int fmtA, int tprRP, const LDesc<T>* d_descs, int ndesc, int maxrows,
                   cudaStream_t s);
 // Gauss-Seidel smoothing phases (levels with nk > 0)

@@ -414,6 +414,16 @@ void launch_phase(int phase, int fmtA, int fmtRP, const LDesc<T>* d_descs, int n
       else
         MGD_DISPATCH_FMT(k_prolong, rp, maxrows, ndesc, s, d_descs);
       break;
+    case PH_POSTQ:
+      switch (fmtRP) {
+        case FMT_CSR2: launch_k(k_postq_csr<T, FMT_CSR2>, dim3(cdiv(2LL * maxrows, kVThreads), ndesc), dim3(kVThreads), 0, s, d_descs); break;
+        case FMT_CSR4: launch_k(k_postq_csr<T, FMT_CSR4>, dim3(cdiv(4LL * maxrows, kVThreads), ndesc), dim3(kVThreads), 0, s, d_descs); break;
+        case FMT_CSR8: launch_k(k_postq_csr<T, FMT_CSR8>, dim3(cdiv(8LL * maxrows, kVThreads), ndesc), dim3(kVThreads), 0, s, d_descs); break;
+        case FMT_CSR16: launch_k(k_postq_csr<T, FMT_CSR16>, dim3(cdiv(16LL * maxrows, kVThreads), ndesc), dim3(kVThreads), 0, s, d_descs); break;
+        case FMT_CSR32: launch_k(k_postq_csr<T, FMT_CSR32>, dim3(cdiv(32LL * maxrows, kVThreads), ndesc), dim3(kVThreads), 0, s, d_descs); break;
+        default: launch_k(k_postq<T>, dim3(cdiv(maxrows, kQWin), ndesc), dim3(kQWin), 0, s, d_descs); break;
+      }
+      break;
     case PH_JAC1: launch_k(k_jac1<T>, dim3(dim3(cdiv(maxrows, kVThreads), ndesc)), dim3(kVThreads), 0, s, d_descs); break;
     case PH_COARSE:
       // one 1024-thread CTA per subsystem: a warp per row of the dense inverse
@@ -434,16 +444,6 @@ template void launch_phase<float>(int, int, int, const LDesc<float>*, int, int, 
 // every point reads only values of other sweeps.  x is the same buffer as xt
 // on these levels.
 template <typename T>
-    case PH_POSTQ:
-      switch (fmtRP) {
-        case FMT_CSR2: launch_k(k_postq_csr<T, FMT_CSR2>, dim3(cdiv(2LL * maxrows, kVThreads), ndesc), dim3(kVThreads), 0, s, d_descs); break;
-        case FMT_CSR4: launch_k(k_postq_csr<T, FMT_CSR4>, dim3(cdiv(4LL * maxrows, kVThreads), ndesc), dim3(kVThreads), 0, s, d_descs); break;
-        case FMT_CSR8: launch_k(k_postq_csr<T, FMT_CSR8>, dim3(cdiv(8LL * maxrows, kVThreads), ndesc), dim3(kVThreads), 0, s, d_descs); break;
-        case FMT_CSR16: launch_k(k_postq_csr<T, FMT_CSR16>, dim3(cdiv(16LL * maxrows, kVThreads), ndesc), dim3(kVThreads), 0, s, d_descs); break;
-        case FMT_CSR32: launch_k(k_postq_csr<T, FMT_CSR32>, dim3(cdiv(32LL * maxrows, kVThreads), ndesc), dim3(kVThreads), 0, s, d_descs); break;
-        default: launch_k(k_postq<T>, dim3(cdiv(maxrows, kQWin), ndesc), dim3(kQWin), 0, s, d_descs); break;
-      }
-      break;
 __global__ void k_gs_first(const LDesc<T>* __restrict__ descs) {
   MGD_PDL_ENTRY();
   const LDesc<T>* d = descs + blockIdx.y;
