@@ -1,0 +1,319 @@
+// arnoldi_kernels.cu -- one FGMRES orthogonalisation (modified Gram-Schmidt of
+// w against the basis, then the normalisation) as one cooperative grid.
+//
+// Modified Gram-Schmidt takes h_i = <v_i, w - sum_{k<i} h_k v_k>, one grid-wide
+// reduction after the other.  With l_ik = <v_i, v_k> the same coefficients
+// solve the unit lower triangular system
+//     h_i + sum_{k<i} l_ik h_k = <v_i, w>
+// (the compact-WY form of modified Gram-Schmidt; Swirydowicz, Langou, Ananthan,
+// Yang, Thomas, "Low synchronization Gram-Schmidt and generalized minimal
+// residual algorithms", Numer. Linear Algebra Appl. 2021), so one pass over the
+// basis gives every <v_i, w>, and with it the new row l_j. of the Gram matrix,
+// and a second pass subtracts sum_i h_i v_i: two grid barriers and 16 bytes per
+// entry of the basis, where a pass per basis vector takes one barrier (or
+// launch) and 32 bytes each.
+//
+// A dot product on the FP64 pipe costs a warp 20 SM clocks per multiply-add
+// here (15.7 G warp instructions/s over 152 SMs), more than the 12 clocks that
+// the 256 bytes it reads take from HBM, and the first pass has two of them per
+// entry.  So that pass multiplies on the integer pipe, exactly: the entries of
+// a unit (32 lanes x K) are aligned to the unit's largest exponent and split
+// into two signed limbs (29 + 29 bits below the largest, a half-unit midpoint
+// for what is cut off), the four limb products are summed in 64-bit integers,
+// folded across the warp as integers, and only the unit's sums become FP64.
+// The rounding against binary64 products is below theirs: 2^-57 of the unit's
+// largest entry per element, of either sign.
+#include "mgd_internal.cuh"
+
+#include <cooperative_groups.h>
+
+namespace mgd {
+
+namespace cg = cooperative_groups;
+
+constexpr int kGsWarps = 12;
+constexpr int kGsThreads = 32 * kGsWarps;
+
+__device__ __forceinline__ int exp_of(int hi) { return (hi >> 20) & 0x7ff; }
+
+// |x| = (53-bit m) 2^(e - 1075) as (h 2^29 + l) 2^(eref - 1082), eref >= e + 2,
+// both limbs with x's sign; l is odd: the midpoint of the cut-off part
+__device__ __forceinline__ void split_limbs(double x, int eref, int& h, int& l) {
+  const int hi = __double2hiint(x);
+  const unsigned r = min((unsigned)(eref - exp_of(hi)), 63u);
+  unsigned long long m = ((unsigned long long)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(x);
+  m = (m << 7) >> r;
+  const int sg = (hi >> 31) | 1;
+  h = (int)(m >> 29) * sg;
+  l = (int)(((unsigned)m & 0x1fffffffu) | 1u) * sg;
+}
+
+// the three sums of a limb dot product, folded over the warp into four 27-bit
+// limbs (the last one signed) of  hh 2^29 + x + ll 2^-29
+struct LimbSum {
+  long long hh = 0, x = 0, ll = 0;
+  __device__ __forceinline__ void add(int ah, int al, int bh, int bl) {
+    hh += (long long)ah * bh;
+    x += (long long)ah * bl;
+    x += (long long)al * bh;
+    ll += (long long)al * bl;
+  }
+  __device__ __forceinline__ int4 fold() const {
+    const __int128 t = ((__int128)hh << 29) + x + (ll >> 29);
+    constexpr unsigned M = (1u << 27) - 1;
+    int4 f;
+    f.x = (int)__reduce_add_sync(0xffffffffu, (unsigned)t & M);
+    f.y = (int)__reduce_add_sync(0xffffffffu, (unsigned)(t >> 27) & M);
+    f.z = (int)__reduce_add_sync(0xffffffffu, (unsigned)(t >> 54) & M);
+    f.w = __reduce_add_sync(0xffffffffu, (int)(t >> 81));
+    return f;
+  }
+};
+
+__device__ __forceinline__ double unfold(const int4& f) {
+  const long long lo = ((long long)(unsigned)f.y << 27) + (unsigned)f.x;
+  const long long hi = ((long long)f.w << 27) + (unsigned)f.z;
+  return fma((double)hi, 0x1p54, (double)lo);
+}
+
+// V: nv basis vectors (leading dimension ldv), each unit's largest biased
+// exponent in vexp[i * nunits + u]; gram: l_ik at gram[k * 32 + i], rows < nv-1
+// given, row nv-1 written by block 0.  Writes h[0..nv-1], *nrm2 = ||w'||^2 and
+// vout = w' / ||w'|| with its exponents; w is only read.
+template <int K>
+__global__ void __launch_bounds__(kGsThreads, 1)
+    k_gram_schmidt(int n, const double* __restrict__ V, long long ldv, int nv, const double* __restrict__ w,
+                   int* vexp, int nunits, double* gram, double* __restrict__ h, double* __restrict__ nrm2,
+                   double* part, double* vout) {
+  __shared__ int4 s_fold[kGsWarps][32][2];
+  __shared__ double s_gram[32 * 32];
+  __shared__ double s_sum[kGsWarps][64];
+  __shared__ double s_dot[64], s_h[32], s_red[kGsWarps];
+  cg::grid_group grid = cg::this_grid();
+  constexpr int U = 32 * K, H = K / 2;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int nb = gridDim.x, gw = blockIdx.x * kGsWarps + warp, nw = nb * kGsWarps;
+  const int j = nv - 1;
+  for (int q = t; q < 32 * 32; q += kGsThreads) s_gram[q] = gram[q];
+
+  // <v_i, w> and <v_i, v_j>, lane i holding those of v_i
+  double acc_w = 0.0, acc_g = 0.0;
+  for (int u = gw; u < nunits; u += nw) {
+    const long long e0 = (long long)u * U + lane;
+    const int ei = lane < nv ? vexp[(size_t)lane * nunits + u] : 0;
+    int ah[K], al[K], bh[K], bl[K];
+    int ew = 0;
+    const int ej = __shfl_sync(0xffffffffu, ei, j);
+    {
+      double x[K], y[K];
+#pragma unroll
+      for (int q = 0; q < K; ++q) {
+        const bool ok = e0 + 32 * q < n;
+        x[q] = ok ? __ldcs(w + e0 + 32 * q) : 0.0;
+        y[q] = ok ? V[(long long)j * ldv + e0 + 32 * q] : 0.0;
+      }
+#pragma unroll
+      for (int q = 0; q < K; ++q) ew = max(ew, exp_of(__double2hiint(x[q])));
+      ew = __reduce_max_sync(0xffffffffu, ew);
+#pragma unroll
+      for (int q = 0; q < K; ++q) {
+        split_limbs(x[q], ew + 2, ah[q], al[q]);
+        if (exp_of(__double2hiint(x[q])) == 0) ah[q] = al[q] = 0;
+        split_limbs(y[q], ej + 2, bh[q], bl[q]);
+        if (exp_of(__double2hiint(y[q])) == 0) bh[q] = bl[q] = 0;
+      }
+    }
+    // (past n these read the next vector or the padding after the basis, times zero limbs of w and v_j)
+    const double* v = V + e0;
+    double va[H], vb[H];
+    auto load = [&](double (&d)[H], int i, int q0) {
+#pragma unroll
+      for (int q = 0; q < H; ++q) d[q] = v[(long long)i * ldv + 32 * (q0 + q)];
+    };
+    load(va, 0, 0);
+    load(vb, 0, H);
+    for (int i = 0; i < nv; ++i) {
+      const int e = __shfl_sync(0xffffffffu, ei, i) + 3;
+      LimbSum dw, dg;
+#pragma unroll
+      for (int q = 0; q < H; ++q) {
+        int vh, vl;
+        split_limbs(va[q], e, vh, vl);
+        dw.add(vh, vl, ah[q], al[q]);
+        dg.add(vh, vl, bh[q], bl[q]);
+      }
+      if (i + 1 < nv) load(va, i + 1, 0);
+#pragma unroll
+      for (int q = 0; q < H; ++q) {
+        int vh, vl;
+        split_limbs(vb[q], e, vh, vl);
+        dw.add(vh, vl, ah[H + q], al[H + q]);
+        dg.add(vh, vl, bh[H + q], bl[H + q]);
+      }
+      if (i + 1 < nv) load(vb, i + 1, H);
+      const int4 fw = dw.fold(), fg = dg.fold();
+      if (lane == 0) {
+        s_fold[warp][i][0] = fw;
+        s_fold[warp][i][1] = fg;
+      }
+    }
+    __syncwarp();
+    if (lane < nv && ei >= 70) {  // a unit of v_i below 2^-953 adds nothing
+      // one unit of the folded sums is 2^(exponents - 2 * 1023 - 84)
+      const double s = 0x1p-84 * __hiloint2double(ei << 20, 0);
+      acc_w += unfold(s_fold[warp][lane][0]) * s * __hiloint2double(ew << 20, 0);
+      acc_g += unfold(s_fold[warp][lane][1]) * s * __hiloint2double(ej << 20, 0);
+    }
+    __syncwarp();
+  }
+  s_sum[warp][lane] = acc_w;
+  s_sum[warp][32 + lane] = acc_g;
+  __syncthreads();
+  if (t < 64 && (t & 31) < nv) {
+    double s = 0.0;
+    for (int q = 0; q < kGsWarps; ++q) s += s_sum[q][t];
+    part[(size_t)t * nb + blockIdx.x] = s;
+  }
+  grid.sync();
+
+  // every block: the dot products from the per-block sums (the same order in
+  // all), then the triangular system, a row per lane
+  for (int p = warp; p < 2 * nv; p += kGsWarps) {
+    const int row = p < nv ? p : 32 + p - nv;
+    double s = 0.0;
+    for (int b = lane; b < nb; b += 32) s += __ldcg(part + (size_t)row * nb + b);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) s_dot[row] = s;
+  }
+  __syncthreads();
+  if (warp == 0) {
+    if (lane < j) s_gram[lane * 32 + j] = s_dot[32 + lane];
+    __syncwarp();
+    double hv = lane < nv ? s_dot[lane] : 0.0;
+    for (int k = 0; k < j; ++k) {
+      const double hk = __shfl_sync(0xffffffffu, hv, k);
+      if (lane > k && lane < nv) hv -= s_gram[k * 32 + lane] * hk;
+    }
+    s_h[lane] = hv;
+    if (blockIdx.x == 0) {
+      if (lane < nv) h[lane] = hv;
+      if (lane < j) gram[lane * 32 + j] = s_gram[lane * 32 + j];
+    }
+  }
+  __syncthreads();
+
+  // w' = w - sum_i h_i v_i and ||w'||^2
+  double ss = 0.0;
+  for (int u = gw; u < nunits; u += nw) {
+    const long long e0 = (long long)u * U + lane;
+    double x[K];
+#pragma unroll
+    for (int q = 0; q < K; ++q) x[q] = e0 + 32 * q < n ? __ldcs(w + e0 + 32 * q) : 0.0;
+#pragma unroll 2
+    for (int i = 0; i < nv; ++i) {
+      const double hi = s_h[i];
+      const double* v = V + (long long)i * ldv + e0;
+#pragma unroll
+      for (int q = 0; q < K; ++q)
+        if (e0 + 32 * q < n) x[q] -= hi * __ldcs(v + 32 * q);
+    }
+#pragma unroll
+    for (int q = 0; q < K; ++q) {
+      ss += x[q] * x[q];
+      if (e0 + 32 * q < n) vout[e0 + 32 * q] = x[q];
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+  if (lane == 0) s_red[warp] = ss;
+  __syncthreads();
+  if (t == 0) {
+    double s = 0.0;
+    for (int q = 0; q < kGsWarps; ++q) s += s_red[q];
+    part[(size_t)64 * nb + blockIdx.x] = s;
+  }
+  grid.sync();
+  double nn = 0.0;  // every warp for itself, in the same order
+  for (int b = lane; b < nb; b += 32) nn += __ldcg(part + (size_t)64 * nb + b);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) nn += __shfl_xor_sync(0xffffffffu, nn, o);
+  if (blockIdx.x == 0 && t == 0) *nrm2 = nn;
+  const double hn = sqrt(nn), inv = hn != 0.0 ? 1.0 / hn : 0.0;
+  // the normalisation, from the units written last (still in L2) to the first
+  const int mine = gw < nunits ? (nunits - 1 - gw) / nw : -1;
+  for (int k = mine; k >= 0; --k) {
+    const int u = gw + k * nw;
+    const long long e0 = (long long)u * U + lane;
+    double x[K];
+    int e = 0;
+#pragma unroll
+    for (int q = 0; q < K; ++q) x[q] = e0 + 32 * q < n ? vout[e0 + 32 * q] * inv : 0.0;
+#pragma unroll
+    for (int q = 0; q < K; ++q) {
+      e = max(e, exp_of(__double2hiint(x[q])));
+      if (e0 + 32 * q < n) vout[e0 + 32 * q] = x[q];
+    }
+    e = __reduce_max_sync(0xffffffffu, e);
+    if (lane == 0) vexp[(size_t)nv * nunits + u] = e;
+  }
+}
+
+// the unit exponents of one vector (a cycle's first basis vector)
+__global__ void __launch_bounds__(kThreads) k_unit_exponents(int n, int unit, const double* __restrict__ v, int* vexp,
+                                                             int nunits) {
+  MGD_PDL_ENTRY();
+  const int u = (blockIdx.x * kThreads + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (u >= nunits) return;
+  const long long e1 = min((long long)n, (long long)(u + 1) * unit);
+  int e = 0;
+  for (long long i = (long long)u * unit + lane; i < e1; i += 32) e = max(e, exp_of(__double2hiint(v[i])));
+  e = __reduce_max_sync(0xffffffffu, e);
+  if (lane == 0) vexp[u] = e;
+}
+
+static const void* gs_kernel(int K) {
+  return K == 2 ? (const void*)k_gram_schmidt<2> : K == 4 ? (const void*)k_gram_schmidt<4>
+       : K == 8 ? (const void*)k_gram_schmidt<8> : (const void*)k_gram_schmidt<16>;
+}
+
+#ifndef MGD_GSK
+#define MGD_GSK 16
+#endif
+GsPlan gs_plan(int n) {
+  GsPlan p;
+  int dev = 0, sms = 0, coop = 0, per = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) ||
+      cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev)) {
+    cudaGetLastError();
+    return p;
+  }
+  if (!coop || sms <= 0 || n <= 0) return p;
+  const long long lanes = (long long)sms * kGsThreads;
+  const int K = n <= 2 * lanes ? 2 : n <= 4 * lanes ? 4 : n <= 8 * lanes ? 8 : MGD_GSK;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, gs_kernel(K), kGsThreads, 0) != cudaSuccess || per < 1) {
+    cudaGetLastError();
+    return p;
+  }
+  p.K = K;
+  p.nunits = cdiv(n, 32 * K);
+  p.nb = std::min(sms, cdiv(p.nunits, kGsWarps));
+  return p;
+}
+
+void launch_unit_exponents(const GsPlan& p, int n, const double* v, int* vexp, cudaStream_t s) {
+  launch_k(k_unit_exponents, dim3(cdiv(32LL * p.nunits, kThreads)), dim3(kThreads), 0, s, n, 32 * p.K, v, vexp,
+           p.nunits);
+  MGD_LAUNCH_CHECK();
+}
+
+void launch_gram_schmidt(const GsPlan& p, int n, const double* V, long long ldv, int nv, const double* w, int* vexp,
+                         double* gram, double* h, double* nrm2, double* part, double* vout, cudaStream_t s) {
+  int nunits = p.nunits;
+  void* args[] = {(void*)&n, (void*)&V, (void*)&ldv, (void*)&nv, (void*)&w, (void*)&vexp, (void*)&nunits,
+                  (void*)&gram, (void*)&h, (void*)&nrm2, (void*)&part, (void*)&vout};
+  MGD_CUDA(cudaLaunchCooperativeKernel(gs_kernel(p.K), dim3(p.nb), dim3(kGsThreads), args, 0, s));
+  MGD_LAUNCH_CHECK();
+}
+
+}  // namespace mgd

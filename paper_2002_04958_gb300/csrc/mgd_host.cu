@@ -1246,7 +1246,9 @@ struct mgd_ctx {
   cudaStream_t s_copy[4] = {nullptr, nullptr, nullptr, nullptr};  // host-to-device copies of mgd_setup_host
   long long graph_kernels = 0;
   long long napply = 0, napplyT = 0; // preconditioner applies since setup (forward, transposed)
-  int arn_nb = 0;                    // blocks of the cooperative Arnoldi grid (0: streaming kernels)
+  mgd::GsPlan gs;                    // the cooperative Gram-Schmidt grid (nb = 0: streaming kernels)
+  int* vexp = nullptr;               // its unit exponents of the basis vectors, and the basis's Gram matrix
+  double* gram = nullptr;
   mgd_stats st;
   int n_jacobi = 0;
   mgd::PhaseClock phases;
@@ -2623,17 +2625,21 @@ static void do_setup(mgd_ctx* c, const int* rp, const int* ci, const double* v, 
   pt_prog.stop();
   PhaseTimer pt_kry(&c->phases, SP_KRYLOV);
   c->m = std::max(1, std::min(o.restart, 30));
-  c->V = c->ar.alloc<double>((size_t)(c->m + 1) * n, true);
-  c->Z = c->ar.alloc<double>((size_t)c->m * n, true);
+  c->V = c->ar.alloc<double>((size_t)(c->m + 1) * n + kGsMaxUnit);  // every vector is written before it is read
+  c->Z = c->ar.alloc<double>((size_t)c->m * n);
   c->w = c->ar.alloc<double>(n, true);
   c->r = c->ar.alloc<double>(n, true);
   c->xtmp = c->ar.alloc<double>(n, true);
   c->btmp = c->ar.alloc<double>(n, true);
   c->hbuf = c->ar.alloc<double>(128, true);
-  c->partial = c->ar.alloc<double>((size_t)kDotBlocks * 32, true);
+  c->gs = o.arnoldi_resident ? gs_plan(n) : GsPlan();
+  c->partial = c->ar.alloc<double>(std::max((size_t)kDotBlocks * 32, (size_t)65 * c->gs.nb), true);
   c->ybuf = c->ar.alloc<double>(64, true);
   if (!c->hpin) MGD_CUDA(cudaMallocHost(&c->hpin, 256 * sizeof(double)));  // kept across setups
-  c->arn_nb = o.arnoldi_resident ? arnoldi_coop_blocks(n) : 0;
+  if (c->gs.nb > 0) {
+    c->vexp = c->ar.alloc<int>((size_t)(c->m + 1) * c->gs.nunits);
+    c->gram = c->ar.alloc<double>(32 * 32, true);
+  }
   // monolithic SpMV layout (cached by operator size, like the V-cycle plans)
   c->fmtMono = FMT_SELL;
   const std::vector<long long> mkey{-1, n, c->A.nnz};
@@ -2788,6 +2794,7 @@ static int fgmres(mgd_ctx* c, const double* b, double* x, double tol, bool trans
     hp[201] = beta * beta;
     MGD_CUDA(cudaMemcpyAsync(c->hbuf + 101, hp + 201, sizeof(double), cudaMemcpyHostToDevice, s));
     launch_scale_by_norm(n, c->r, c->hbuf + 101, c->V, s);
+    if (c->gs.nb > 0) launch_unit_exponents(c->gs, n, c->V, c->vexp, s);
     std::fill(g.begin(), g.end(), 0.0);
     g[0] = beta;
     int j = 0;
@@ -2800,8 +2807,8 @@ static int fgmres(mgd_ctx* c, const double* b, double* x, double tol, bool trans
       int nv = j + 1;
       int aid = c->prof.begin(s, 3);
       // modified Gram-Schmidt: h in hbuf[0..j], ||w||^2 in hbuf[64], v_{j+1} = w / ||w||
-      if (c->arn_nb > 0) {
-        launch_arnoldi_coop(c->arn_nb, n, c->V, n, nv, c->w, c->hbuf, c->hbuf + 64, c->partial,
+      if (c->gs.nb > 0) {
+        launch_gram_schmidt(c->gs, n, c->V, n, nv, c->w, c->vexp, c->gram, c->hbuf, c->hbuf + 64, c->partial,
                             c->V + (size_t)(j + 1) * n, s);
       } else {
         // class 5: the j+1 fused Gram-Schmidt steps alone (32 n bytes each)
@@ -2812,7 +2819,9 @@ static int fgmres(mgd_ctx* c, const double* b, double* x, double tol, bool trans
         // the last step (index nv-1) ran backwards when nv-1 is odd: run the opposite way
         launch_scale_by_norm(n, c->w, c->hbuf + 64, c->V + (size_t)(j + 1) * n, s, ((nv - 1) & 1) ? 0 : 1);
       }
-      c->prof.end(aid, 3, 8.0 * n * (4.0 * nv + 2.0 + 2.0), s);
+      // cooperative: the basis twice, w twice, v_j, w' out, in and out again; streaming: 4 n a step, the first dot
+      // product and the scaling
+      c->prof.end(aid, 3, 8.0 * n * (c->gs.nb > 0 ? 2.0 * nv + 5.0 : 4.0 * nv + 2.0 + 2.0), s);
       MGD_CUDA(cudaMemcpyAsync(hp, c->hbuf, 65 * sizeof(double), cudaMemcpyDeviceToHost, s));
       MGD_CUDA(cudaStreamSynchronize(s));
       c->prof.harvest();

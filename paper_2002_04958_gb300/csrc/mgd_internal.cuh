@@ -613,12 +613,17 @@ void launch_mgs(int n, const double* V, long long ldv, int nv, double* w, double
 // rev: traverse the vectors backwards (the streaming Arnoldi alternates
 // directions between passes; 1 after a launch_mgs whose last step ran forwards)
 void launch_scale_by_norm(int n, const double* w, const double* nrm2, double* v, cudaStream_t s, int rev = 0);
-// the same modified Gram-Schmidt pass plus the scaling, as one cooperative
-// grid of nb blocks with w in shared memory (nb from arnoldi_coop_blocks; part:
-// (nv + 1) * nb doubles)
-int arnoldi_coop_blocks(int n);
-void launch_arnoldi_coop(int nb, int n, const double* V, long long ldv, int nv, const double* w, double* h,
-                         double* nrm2, double* part, double* vout, cudaStream_t s);
+// the same Gram-Schmidt pass plus the scaling as one cooperative grid (arnoldi_kernels.cu):
+// units of 32 K entries, nunits of them, nb blocks (0: not available)
+struct GsPlan {
+  int K = 0, nunits = 0, nb = 0;
+};
+constexpr int kGsMaxUnit = 512;  // entries that may be read past the last basis vector
+GsPlan gs_plan(int n);
+// vexp: (restart + 1) * nunits ints; gram: 1024 doubles; part: 65 * nb doubles; V has kGsMaxUnit entries after it
+void launch_unit_exponents(const GsPlan& p, int n, const double* v, int* vexp, cudaStream_t s);
+void launch_gram_schmidt(const GsPlan& p, int n, const double* V, long long ldv, int nv, const double* w, int* vexp,
+                         double* gram, double* h, double* nrm2, double* part, double* vout, cudaStream_t s);
 void launch_vcomb(int n, const double* Z, long long ldz, int nv, const double* y, double* x, cudaStream_t s);
 void launch_norm2(int n, const double* x, double* partial, double* out, cudaStream_t s);
 void launch_block_resid(int N, int nc, const int* const* brp, const int* const* bci, const double* const* bv,

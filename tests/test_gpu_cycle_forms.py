@@ -77,3 +77,43 @@ def test_q_layouts_match_oracle(gpu, orc, tmp_path):
         if f in (0, 1, 9, 10):  # the same kernel
             same = same or got
             assert all(np.array_equal(a, b) for a, b in zip(got, same)), f
+
+
+# unknowns at which the Gram-Schmidt grid's units grow (116,736, 233,472 and 466,944 on 152 SMs), on either side, and
+# the smallest: fewer than a unit, one block, a last unit of one entry
+GS_GRIDS = [(3, 3), (64, 32), (11, 31), (512, 76), (357, 109), (304, 256), (275, 283), (512, 304), (395, 395)]
+
+
+@pytest.mark.parametrize("dims", GS_GRIDS, ids=["x".join(map(str, d)) for d in GS_GRIDS])
+def test_gram_schmidt_grid_matches_streaming(gpu, dims):
+    # both orthogonalise by modified Gram-Schmidt, to rounding; right-hand sides: dense, one cell, and a
+    # scale far from one with a decay over 13 orders of magnitude
+    import torch
+    s = inputs.make_system(1, dims, multigroup=True)
+    rng = np.random.default_rng(5)
+    point = np.zeros(s.n)
+    point[s.n // 2] = 1.0
+    grid = gpu.Solver(autotune=0, arnoldi_resident=1).setup_system(s, "schur1")
+    stream = gpu.Solver(autotune=0, arnoldi_resident=0).setup_system(s, "schur1")
+    for b in (s.b, point, 1e100 * np.exp(-30.0 * np.arange(s.n) / s.n) * rng.standard_normal(s.n)):
+        b = torch.from_numpy(b)
+        xg, itg, rg, _ = grid.solve(b)
+        xs, its, rs, _ = stream.solve(b)
+        assert itg == its
+        assert torch.linalg.vector_norm(xg - xs) <= 1e-10 * torch.linalg.vector_norm(xs)
+        assert np.allclose(grid.history(), stream.history(), rtol=1e-4, atol=1e-13)
+
+
+def test_gram_schmidt_grid_not_finite(gpu):
+    # an infinity or a NaN in the right-hand side ends the solve with its status, as it did
+    import torch
+    s = inputs.make_system(1, (64, 32), multigroup=True)
+    slv = gpu.Solver(autotune=0).setup_system(s, "schur1")
+    for bad in (np.inf, np.nan):
+        b = s.b.copy()
+        b[777] = bad
+        with pytest.raises(gpu.MgdError) as e:
+            slv.solve(torch.from_numpy(b))
+        assert e.value.code == 5
+    x, it, rr, rc = slv.solve(torch.from_numpy(s.b))
+    assert rc == 0 and rr <= 1e-8
