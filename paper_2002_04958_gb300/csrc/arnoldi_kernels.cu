@@ -23,6 +23,12 @@
 // folded across the warp as integers, and only the unit's sums become FP64.
 // The rounding against binary64 products is below theirs: 2^-57 of the unit's
 // largest entry per element, of either sign.
+//
+// Measured per call with 16 vectors, against the streaming kernels: 3,072
+// unknowns 20.5 / 110.9 us, 148,074 33 / 178 us, 3.1 M 227 / 394 us, 19.5 M
+// 1160 / 1617 us; there the first pass takes 23 us a vector (its 156 MB at the
+// copy bandwidth) and the second 39 us, its FP64 issue slots.  The second pass
+// on the integer pipe was no faster (34 us a vector, and more per call).
 #include "mgd_internal.cuh"
 
 #include <cooperative_groups.h>
@@ -33,6 +39,7 @@ namespace cg = cooperative_groups;
 
 constexpr int kGsWarps = 12;
 constexpr int kGsThreads = 32 * kGsWarps;
+constexpr int kGsMinWarps = 8;  // busy warps to a block before there is another block
 
 __device__ __forceinline__ int exp_of(int hi) { return (hi >> 20) & 0x7ff; }
 
@@ -83,22 +90,26 @@ __device__ __forceinline__ double unfold(const int4& f) {
 template <int K>
 __global__ void __launch_bounds__(kGsThreads, 1)
     k_gram_schmidt(int n, const double* __restrict__ V, long long ldv, int nv, const double* __restrict__ w,
-                   int* vexp, int nunits, double* gram, double* __restrict__ h, double* __restrict__ nrm2,
-                   double* part, double* vout) {
+                   int* vexp, int nunits, int share_of_short, double* gram, double* __restrict__ h,
+                   double* __restrict__ nrm2, double* part, double* vout) {
   __shared__ int4 s_fold[kGsWarps][32][2];
   __shared__ double s_gram[32 * 32];
   __shared__ double s_sum[kGsWarps][64];
   __shared__ double s_dot[64], s_h[32], s_red[kGsWarps];
   cg::grid_group grid = cg::this_grid();
-  constexpr int U = 32 * K, H = K / 2;
+  constexpr int U = 32 * K, H = K / 2, UI = K >= 16 ? 2 : K >= 8 ? 4 : 8;
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  const int nb = gridDim.x, gw = blockIdx.x * kGsWarps + warp, nw = nb * kGsWarps;
+  // warps are numbered across the blocks, so that units spread over all SMs
+  const int nb = gridDim.x, gw = warp * nb + blockIdx.x, nw = nb * kGsWarps;
   const int j = nv - 1;
   for (int q = t; q < 32 * 32; q += kGsThreads) s_gram[q] = gram[q];
 
-  // <v_i, w> and <v_i, v_j>, lane i holding those of v_i
+  // <v_i, w> and <v_i, v_j>, lane i holding those of v_i; `share` warps take a
+  // unit, each every share-th vector
   double acc_w = 0.0, acc_g = 0.0;
-  for (int u = gw; u < nunits; u += nw) {
+  const int share = K <= 4 ? share_of_short : 1;
+  const int i0 = gw % share;
+  for (int u = gw / share; u < nunits; u += nw / share) {
     const long long e0 = (long long)u * U + lane;
     const int ei = lane < nv ? vexp[(size_t)lane * nunits + u] : 0;
     int ah[K], al[K], bh[K], bl[K];
@@ -130,27 +141,27 @@ __global__ void __launch_bounds__(kGsThreads, 1)
 #pragma unroll
       for (int q = 0; q < H; ++q) d[q] = v[(long long)i * ldv + 32 * (q0 + q)];
     };
-    load(va, 0, 0);
-    load(vb, 0, H);
-    for (int i = 0; i < nv; ++i) {
+    auto take = [&](const double (&d)[H], int i, int q0, LimbSum& dw, LimbSum& dg) {
       const int e = __shfl_sync(0xffffffffu, ei, i) + 3;
+#pragma unroll
+      for (int q = 0; q < H; ++q) {
+        int vh, vl;
+        split_limbs(d[q], e, vh, vl);
+        dw.add(vh, vl, ah[q0 + q], al[q0 + q]);
+        dg.add(vh, vl, bh[q0 + q], bl[q0 + q]);
+      }
+    };
+    if (i0 < nv) {
+      load(va, i0, 0);
+      load(vb, i0, H);
+    }
+#pragma unroll 1
+    for (int i = i0; i < nv; i += share) {
       LimbSum dw, dg;
-#pragma unroll
-      for (int q = 0; q < H; ++q) {
-        int vh, vl;
-        split_limbs(va[q], e, vh, vl);
-        dw.add(vh, vl, ah[q], al[q]);
-        dg.add(vh, vl, bh[q], bl[q]);
-      }
-      if (i + 1 < nv) load(va, i + 1, 0);
-#pragma unroll
-      for (int q = 0; q < H; ++q) {
-        int vh, vl;
-        split_limbs(vb[q], e, vh, vl);
-        dw.add(vh, vl, ah[H + q], al[H + q]);
-        dg.add(vh, vl, bh[H + q], bl[H + q]);
-      }
-      if (i + 1 < nv) load(vb, i + 1, H);
+      take(va, i, 0, dw, dg);
+      if (i + share < nv) load(va, i + share, 0);
+      take(vb, i, H, dw, dg);
+      if (i + share < nv) load(vb, i + share, H);
       const int4 fw = dw.fold(), fg = dg.fold();
       if (lane == 0) {
         s_fold[warp][i][0] = fw;
@@ -158,7 +169,7 @@ __global__ void __launch_bounds__(kGsThreads, 1)
       }
     }
     __syncwarp();
-    if (lane < nv && ei >= 70) {  // a unit of v_i below 2^-953 adds nothing
+    if (lane < nv && lane % share == i0 && ei >= 70) {  // a unit of v_i below 2^-953 adds nothing
       // one unit of the folded sums is 2^(exponents - 2 * 1023 - 84)
       const double s = 0x1p-84 * __hiloint2double(ei << 20, 0);
       acc_w += unfold(s_fold[warp][lane][0]) * s * __hiloint2double(ew << 20, 0);
@@ -210,7 +221,7 @@ __global__ void __launch_bounds__(kGsThreads, 1)
     double x[K];
 #pragma unroll
     for (int q = 0; q < K; ++q) x[q] = e0 + 32 * q < n ? __ldcs(w + e0 + 32 * q) : 0.0;
-#pragma unroll 2
+#pragma unroll UI
     for (int i = 0; i < nv; ++i) {
       const double hi = s_h[i];
       const double* v = V + (long long)i * ldv + e0;
@@ -277,9 +288,6 @@ static const void* gs_kernel(int K) {
        : K == 8 ? (const void*)k_gram_schmidt<8> : (const void*)k_gram_schmidt<16>;
 }
 
-#ifndef MGD_GSK
-#define MGD_GSK 16
-#endif
 GsPlan gs_plan(int n) {
   GsPlan p;
   int dev = 0, sms = 0, coop = 0, per = 0;
@@ -290,14 +298,22 @@ GsPlan gs_plan(int n) {
   }
   if (!coop || sms <= 0 || n <= 0) return p;
   const long long lanes = (long long)sms * kGsThreads;
-  const int K = n <= 2 * lanes ? 2 : n <= 4 * lanes ? 4 : n <= 8 * lanes ? 8 : MGD_GSK;
+  // long units fold less often, short ones keep every warp busy: the shortest
+  // that still gives each warp one unit, then 256 entries while 512 would leave
+  // a warp five or fewer (1 M unknowns, 16 vectors: 100 us against 128 us;
+  // 19.5 M: 1280 against 1160)
+  const int K = n <= 2 * lanes ? 2 : n <= 4 * lanes ? 4 : n <= 80 * lanes ? 8 : 16;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, gs_kernel(K), kGsThreads, 0) != cudaSuccess || per < 1) {
     cudaGetLastError();
     return p;
   }
   p.K = K;
   p.nunits = cdiv(n, 32 * K);
-  p.nb = std::min(sms, cdiv(p.nunits, kGsWarps));
+  // a short vector leaves warps without a unit: several share one (3,072
+  // unknowns, 30 vectors: 35 -> 25 us)
+  p.share = 1;
+  while (K <= 4 && p.share < 8 && (long long)p.nunits * p.share * 2 <= (long long)sms * kGsWarps) p.share *= 2;
+  p.nb = std::min(sms, cdiv((long long)p.nunits * p.share, kGsMinWarps));
   return p;
 }
 
@@ -309,9 +325,9 @@ void launch_unit_exponents(const GsPlan& p, int n, const double* v, int* vexp, c
 
 void launch_gram_schmidt(const GsPlan& p, int n, const double* V, long long ldv, int nv, const double* w, int* vexp,
                          double* gram, double* h, double* nrm2, double* part, double* vout, cudaStream_t s) {
-  int nunits = p.nunits;
+  int nunits = p.nunits, share = p.share;
   void* args[] = {(void*)&n, (void*)&V, (void*)&ldv, (void*)&nv, (void*)&w, (void*)&vexp, (void*)&nunits,
-                  (void*)&gram, (void*)&h, (void*)&nrm2, (void*)&part, (void*)&vout};
+                  (void*)&share, (void*)&gram, (void*)&h, (void*)&nrm2, (void*)&part, (void*)&vout};
   MGD_CUDA(cudaLaunchCooperativeKernel(gs_kernel(p.K), dim3(p.nb), dim3(kGsThreads), args, 0, s));
   MGD_LAUNCH_CHECK();
 }
