@@ -88,7 +88,9 @@ typedef struct mgd_opts {
   int keep_transpose;     /* 1: keep A_l^T per level so that mgd_solve_transpose can run */
   int fuse_rows;          /* levels below level 0 whose subsystems all have <= fuse_rows rows run, with every
                              coarser level, in one thread-block-cluster launch per V-cycle; 0: chosen by the
-                             autotuner (not fused when autotune is off); -1: never */
+                             autotuner, which may also form the cycle from a level of at most 2048 rows down as
+                             one dense matrix per subsystem at setup and apply that (not fused when autotune is
+                             off); -1: never */
   int interp_type;        /* 0: classical modified interpolation (Section 3.1); 1: extended+i (distance-two
                              classical interpolation, De Sterck, Falgout, Nolting, Yang 2008) */
   int pdl;                /* 1: solve kernels use programmatic dependent launch (each waits on its predecessor
@@ -108,9 +110,9 @@ typedef struct mgd_opts {
                              PMIS pass (weight stream 1100 + level) on A1 = P1^T A P1, which is not kept as a
                              level, chooses the final C points among the first pass's; P = P1 P2 (two-stage
                              interpolation, each stage of interp_type).  0: none (default); at most max_levels */
-  int arnoldi_resident;   /* 1 (default): each FGMRES orthogonalisation runs as one cooperative grid that keeps the
-                             new Krylov vector in shared memory (one block per SM; used when n fits, else 0);
-                             0: one streaming kernel per basis vector.  Same modified Gram-Schmidt either way */
+  int arnoldi_resident;   /* 1 (default): each FGMRES orthogonalisation runs as one cooperative grid that reads the
+                             basis twice (0 where the device has no cooperative launch); 0: one streaming kernel
+                             per basis vector.  Modified Gram-Schmidt coefficients either way */
   int opt4_steps;         /* option #4 (Section 3.5).  0 (default): off.  K in 1..1000: the Schur complement
                              whose inner inverse is one block -- S_I = A_I - D_IE A_E^-1 D_EI of Schur2 and
                              C_E = A_E - D_EI A_I^-1 D_IE of Schur1 -- is inverted by K steps of
@@ -256,7 +258,10 @@ int mgd_setup_phases(mgd_ctx *c, double *h_ms, int n);
  * (0 = SELL-32, 1..6 = CSR with 1, 2, 4, 8, 16, 32 threads per row, 7 / 8 =
  * SELL-32 with a thread on 2 / 4 slices, 9 / 10 = CSR with a thread on one
  * row of each of 2 / 4 adjacent 32-row groups); *tail =
- * first level handled by the fused coarse-level kernel (depth if none). */
+ * first level handled by the fused coarse-level kernel or the dense coarse
+ * cycle (depth if none).  On l1-Jacobi levels fmtP is the layout of the
+ * combined prolongation and post-smoothing: 0, 1, 9 and 10 its length-sorted
+ * SELL-32, 2..6 CSR with 2, 4, 8, 16, 32 threads per row. */
 int mgd_plan_info(mgd_ctx *c, int batch, int level, int *nbatches, int *depth, int *nsub, int *maxrows, int *fmtA,
                   int *fmtR, int *fmtP, int *tail);
 
@@ -272,17 +277,19 @@ int mgd_plan_info(mgd_ctx *c, int batch, int level, int *nbatches, int *depth, i
  * class 0, i.e. every V-cycle kernel), the launch count, the summed device
  * time and the summed algorithmic bytes.  V-cycle launches are also counted
  * under detail classes: 16 + 4*level + phase (phase 0 pre-smoothing +
- * residual, 1 restriction, 2 prolongation, 3 post-smoothing), 400 + level for
- * coarsest-level solves, 15 for the fused coarse-level kernel.  With opts.use_graph the selected
+ * residual, 1 restriction, 2 prolongation (Gauss-Seidel levels and transposed
+ * cycles; elsewhere it is part of phase 3), 3 post-smoothing), 400 + level for
+ * coarsest-level solves, 15 for the fused or dense coarse levels.  With opts.use_graph the selected
  * kernels are bracketed by event nodes inside the captured graph (the graph is
  * captured again when the mask changes), so timing does not change how the
  * preconditioner is launched. */
 int mgd_profile_enable(mgd_ctx *c, int mask);
 int mgd_profile_read(mgd_ctx *c, int cls, long long *launches, double *ms, double *bytes);
 /* The algorithmic FP64 lane operations of the launches class cls recorded
- * (same classes and synchronisation as mgd_profile_read): one per nonzero and
- * two per row for the l1-Jacobi smoothing + residual kernels (k_pre, k_post),
- * one more per row for a stalled coarsest level's first sweep; zero for
+ * (same classes and synchronisation as mgd_profile_read): one per nonzero of A
+ * and two per row for the l1-Jacobi smoothing + residual kernels on the way
+ * down and for the smoothing on the way up (the method's operations, also
+ * where the way up runs as one product with P - D^-1 A P), one more per row for a stalled coarsest level's first sweep; zero for
  * FP32 V-cycles, Gauss-Seidel levels and the other kernels.  Together with
  * mgd_fp64_issue_rate it places the level-0 kernels against the FP64 issue
  * limit, which on GB300 is as low as the HBM limit for one multiply-add per

@@ -698,6 +698,16 @@ static void build_hierarchy(SetupCtx& sc, Hier& h, const Csr& A0) {
 }
 
 // ------------------------------------------------------------------ batched V-cycle plans
+// tail_cs of a batch whose levels from tail_level down are one dense matrix
+// per subsystem (stored in tuning files beside the cluster sizes 8 and 16)
+constexpr int kTailDense = 1;
+// largest matrix, and the most entries of a batch's matrices together, that
+// the tuner offers (32 MB: some 8 us of FP64 issue slots and of reads); it
+// times the first levels below 1/64, 1/8 and all of that against no dense
+// level, since what a dense level replaces depends on depth and smoother
+constexpr int kDenseMaxRows = 2048;
+constexpr double kDenseMaxEntries = 4 << 20;
+
 template <typename T>
 struct VBatch {
   std::vector<Hier*> hs;
@@ -727,7 +737,10 @@ struct VBatch {
   // fused coarse-level kernel: levels >= tail_level of every subsystem in one
   // cluster launch (tail_level >= depth: not used)
   int tail_level = 1 << 20;
-  int tail_cs = 8;
+  int tail_cs = 8;  // cluster size, or kTailDense: one dense product per subsystem instead
+  LDesc<T>* d_dense = nullptr;
+  LDesc<T>* d_denseT = nullptr;
+  int dense_maxn = 0;
   TailSub<T>* d_tail = nullptr;
   TailSub<T>* d_tailT = nullptr;
   int ntail = 0;
@@ -934,7 +947,9 @@ static void run_vbatch(VBatch<T>& vb, bool trans, cudaStream_t s, Profiler& prof
   if (tail) {
     prof.next_detail = 15;
     int id = prof.begin(s, 1);
-    launch_vtail<T>(trans ? vb.d_tailT : vb.d_tail, vb.ntail, vb.tail_cs, s);
+    if (vb.tail_cs == kTailDense)
+      launch_phase<T>(PH_COARSE, FMT_SELL, FMT_CSR1, trans ? vb.d_denseT : vb.d_dense, vb.ntail, vb.dense_maxn, s);
+    else launch_vtail<T>(trans ? vb.d_tailT : vb.d_tail, vb.ntail, vb.tail_cs, s);
     prof.end(id, 1, vb.tail_bytes, s);
   }
   for (int l = std::min(vb.depth - 2, ltop - 1); l >= 0; --l) {
@@ -988,6 +1003,94 @@ static void build_tail(Arena& ar, VBatch<T>& vb, int Lt, bool keepT, cudaStream_
     vb.tail_bytes += lp.bytes_pre + lp.bytes_post + lp.bytes_restrict + lp.bytes_prolong + lp.bytes_coarse +
                      lp.bytes_jac + lp.bytes_post_cj;
   }
+}
+
+// Dense form of the levels from Lt (>= 1) down: each subsystem's cycle matrix
+// (its transpose is the transposed cycle), or its coarsest inverse where Lt is
+// that level.  The matrices are formed on the context stream.
+template <typename T>
+static void build_dense(Arena& ar, VBatch<T>& vb, int Lt, bool keepT, cudaStream_t s) {
+  vb.tail_level = std::min(Lt, vb.depth);
+  vb.tail_cs = kTailDense;
+  vb.ntail = 0;
+  vb.tail_bytes = 0;
+  vb.dense_maxn = 0;
+  if (Lt >= vb.depth) return;
+  std::vector<LDesc<double>> lev;  // the levels of the subsystems with a matrix to form, one after the other
+  std::vector<CycSub> subs;
+  std::vector<size_t> first;
+  std::vector<LDesc<T>> desc[2];
+  int blocks = 0;
+  size_t wsn = 0;
+  for (Hier* h : vb.hs) {
+    if (h->nlev() <= Lt) continue;
+    const int n = h->L[Lt].A.n;
+    const bool inverse = h->nlev() == Lt + 1 && h->coarse_lu;
+    CycSub c;
+    memset(&c, 0, sizeof(c));
+    if (!inverse) {
+      c.out = ar.alloc<double>((size_t)n * n);
+      if (keepT) c.outT = ar.alloc<double>((size_t)n * n);
+      c.nlev = h->nlev() - Lt;
+      c.coarse_lu = h->coarse_lu ? 1 : 0;
+      first.push_back(lev.size());
+      for (int l = Lt; l < h->nlev(); ++l) {
+        lev.push_back(make_desc<double>(*h, l, false));
+        c.rows += h->L[l].A.n;
+      }
+      c.blk0 = blocks;
+      c.ws0 = wsn;
+      blocks += cdiv(n, kCycCols);
+      wsn += (size_t)cdiv(n, kCycCols) * kCycCols * kCycVecs * c.rows;
+      subs.push_back(c);
+    }
+    for (int t = 0; t < (keepT ? 2 : 1); ++t) {
+      LDesc<T> d = make_desc<T>(*h, Lt, t == 1);
+      if (!inverse) d.cinv = t ? c.outT : c.out;
+      d.cn = n;
+      desc[t].push_back(d);
+    }
+    ++vb.ntail;
+    vb.dense_maxn = std::max(vb.dense_maxn, n);
+    vb.tail_bytes += 8.0 * n * n + 2.0 * sizeof(T) * n;
+  }
+  if (!vb.ntail) return;
+  auto upload = [&](const auto& v) {
+    using D = typename std::decay_t<decltype(v)>::value_type;
+    D* p = ar.alloc<D>(v.size());
+    MGD_CUDA(cudaMemcpyAsync(p, v.data(), sizeof(D) * v.size(), cudaMemcpyHostToDevice, s));
+    return p;
+  };
+  vb.d_dense = upload(desc[0]);
+  if (keepT) vb.d_denseT = upload(desc[1]);
+  if (blocks > 0) {
+    const LDesc<double>* dl = upload(lev);
+    for (size_t i = 0; i < subs.size(); ++i) subs[i].lev = dl + first[i];
+    CycSub end;
+    memset(&end, 0, sizeof(end));
+    end.blk0 = blocks;
+    subs.push_back(end);
+    Scratch sc(s, ar.pool);
+    launch_cycle_columns(upload(subs), blocks, sc.alloc<double>(wsn), s);
+  }
+  MGD_CUDA(cudaStreamSynchronize(s));  // host vectors above go out of scope
+}
+
+// first level >= 1 whose matrices fit the bounds (vb.depth: none)
+template <typename T>
+static int dense_level(const VBatch<T>& vb, double max_entries) {
+  for (int l = 1; l < vb.depth; ++l) {
+    double e = 0;
+    bool ok = true;
+    for (Hier* h : vb.hs)
+      if (h->nlev() > l) {
+        const double n = h->L[l].A.n;
+        e += n * n;
+        ok = ok && n <= kDenseMaxRows;
+      }
+    if (ok && e <= max_entries) return l;
+  }
+  return vb.depth;
 }
 
 // Autotune the first fused level: time whole V-cycles with no fusion and with
@@ -1064,10 +1167,24 @@ static void autotune_tail(Arena& ar, VBatch<T>& vb, bool keepT, bool graph, cuda
       }
     }
   }
+  std::vector<int> tried;
+  for (double e : {kDenseMaxEntries / 64, kDenseMaxEntries / 8, kDenseMaxEntries}) {
+    const int Lt = dense_level(vb, e);
+    if (Lt >= vb.depth || std::find(tried.begin(), tried.end(), Lt) != tried.end()) continue;
+    tried.push_back(Lt);
+    build_dense<T>(ar, vb, Lt, keepT, s);
+    float ms = time_cycles();
+    if (ms < best) {
+      best = ms;
+      best_lt = Lt;
+      best_cs = kTailDense;
+    }
+  }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   vb.tail_cs = best_cs;
-  build_tail<T>(ar, vb, best_lt, keepT, s);
+  if (best_cs == kTailDense) build_dense<T>(ar, vb, best_lt, keepT, s);
+  else build_tail<T>(ar, vb, best_lt, keepT, s);
 }
 
 // Autotuner: per level of a batch, time the operator phase (PRE) under each
@@ -2200,7 +2317,12 @@ static void build_batches(mgd_ctx* c) {
     }
     if (cached) {
       vb.tail_cs = g_tune_cache[key].tail_cs;
-      build_tail<T>(c->ar, vb, g_tune_cache[key].tail_level, c->o.keep_transpose != 0, c->s);
+      const int Lt = g_tune_cache[key].tail_level;
+      // the file may hold a level whose matrices are over the bounds here
+      if (vb.tail_cs == kTailDense && Lt >= std::max(1, dense_level(vb, kDenseMaxEntries)))
+        build_dense<T>(c->ar, vb, Lt, c->o.keep_transpose != 0, c->s);
+      else
+        build_tail<T>(c->ar, vb, vb.tail_cs == kTailDense ? vb.depth : Lt, c->o.keep_transpose != 0, c->s);
       continue;
     }
     if (c->o.autotune) {

@@ -336,7 +336,8 @@ struct LDesc {
   T* r;   // residual
   T* bc;  // next level's right-hand side
   T* xc;  // next level's output
-  // coarsest level: dense inverse (FP64, row-major cn x cn)
+  // a level solved by one dense product x = cinv b (FP64, row-major cn x cn):
+  // the coarsest level's inverse, or the whole cycle from this level down
   const double* cinv;
   int cn;
   // option #3 / multi-cycle loops: the subsystem's flag (nullptr: always
@@ -370,6 +371,17 @@ struct TailSub {
   const LDesc<T>* lev;  // device array, nlev entries (first = first fused level)
   int nlev;             // fused levels including the coarsest (>= 1)
   int coarse_lu;        // coarsest: 1 dense inverse, 0 two l1-Jacobi sweeps
+};
+
+// k_cycle_columns: blocks of kCycCols unit vectors, kCycVecs work vectors per level
+constexpr int kCycCols = 32, kCycVecs = 3;
+struct CycSub {               // one subsystem's cycle matrix
+  const LDesc<double>* lev;   // its levels from the one whose cycle is formed (FP64 arrays)
+  int nlev, coarse_lu;
+  int blk0;                   // its first block (the list ends with one whose blk0 is the grid size)
+  size_t rows, ws0;           // rows of all its levels; its first element of the workspace
+  double* out;                // out[r * n + c] = (V e_c)_r, n = lev[0].n
+  double* outT;               // the transpose, or nullptr
 };
 
 // Block-level pointer reference: absolute, or relative to the current
@@ -558,6 +570,8 @@ void launch_gs_resid(int fmtA, const LDesc<T>* d, int nd, int maxrows, cudaStrea
 template <typename T>
 void launch_vtail(const TailSub<T>* d_subs, int nsub, int cs, cudaStream_t s);
 constexpr int kTailThreads = 512;
+// the cycle matrices of d_subs: nblocks blocks, ws with kCycCols * kCycVecs * rows doubles for each block
+void launch_cycle_columns(const CycSub* d_subs, int nblocks, double* ws, cudaStream_t s);
 template <typename T>
 bool vtail_cluster_fits(int cs);
 

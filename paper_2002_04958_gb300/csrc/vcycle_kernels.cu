@@ -334,25 +334,68 @@ __global__ void k_jac1(const LDesc<T>* __restrict__ descs) {
   if (i < d->n) d->xt[i] = d->dinv[i] * d->b[i];
 }
 
-// coarsest level: x = A_L^{-1} b with the dense FP64 inverse (one CTA per subsystem)
-template <typename T>
-__global__ void k_coarse(const LDesc<T>* __restrict__ descs) {
-  MGD_PDL_ENTRY();
+// x = M b for a dense FP64 matrix per subsystem: the coarsest level's inverse,
+// or the cycle from a coarse level down (k_cycle_columns).  At these sizes
+// latency is the time: the matrix entries a lane needs first are loaded before
+// the dependency wait.  A warp takes R rows: one where there are few (more
+// SMs share the reads and the FP64 issue slots), four where the chip is full
+// anyway (their sums are folded across the lanes together, 6 FP64 additions
+// for four rows instead of 20).
+constexpr int kDenseThreads = 128;
+template <typename T, int R>
+__global__ void __launch_bounds__(kDenseThreads) k_coarse(const LDesc<T>* __restrict__ descs) {
+  static_assert(R == 1 || R == 4, "the folding below");
+  constexpr int PRE = R == 1 ? 8 : 3;
+  MGD_PDL_TRIGGER();
   const LDesc<T>* d = descs + blockIdx.y;
-  MGD_SKIP_INACTIVE(d);
-  extern __shared__ double sb[];
-  int n = d->cn;
-  for (int j = threadIdx.x; j < n; j += blockDim.x) sb[j] = (double)d->b[j];
-  __syncthreads();
-  int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  for (int i = warp; i < n; i += nw) {
-    const double* row = d->cinv + (size_t)i * n;
-    double s = 0.0;
-    for (int j = lane; j < n; j += 32) s += row[j] * sb[j];
+  const int n = d->cn;
+  const int lane = threadIdx.x & 31;
+  const int i0 = (blockIdx.x * (kDenseThreads / 32) + (threadIdx.x >> 5)) * R;
+  if (i0 >= n) return;
+  const double* m = d->cinv + (size_t)i0 * n;
+  double pre[R][PRE], s[R];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) d->x[i] = (T)s;
+  for (int q = 0; q < R; ++q) {
+    s[q] = 0.0;
+#pragma unroll
+    for (int p = 0; p < PRE; ++p)
+      pre[q][p] = i0 + q < n && lane + 32 * p < n ? __ldg(m + (size_t)q * n + lane + 32 * p) : 0.0;
   }
+  MGD_PDL_WAIT();
+  MGD_SKIP_INACTIVE(d);
+  const T* b = d->b;
+#pragma unroll
+  for (int p = 0; p < PRE; ++p)
+    if (lane + 32 * p < n) {
+      const double bj = (double)__ldg(b + lane + 32 * p);
+#pragma unroll
+      for (int q = 0; q < R; ++q) s[q] += pre[q][p] * bj;
+    }
+#pragma unroll 4
+  for (int j = lane + 32 * PRE; j < n; j += 32) {
+    const double bj = (double)__ldg(b + j);
+#pragma unroll
+    for (int q = 0; q < R; ++q)
+      if (i0 + q < n) s[q] += __ldg(m + (size_t)q * n + j) * bj;
+  }
+  double t;
+  int i = i0;
+  if constexpr (R == 1) {
+    t = s[0];
+#pragma unroll
+    for (int o = 16; o > 4; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  } else {  // lanes 0-15 take rows 0 and 1, the others 2 and 3, then each half of those one row
+    const bool hi = lane & 16, hi2 = lane & 8;
+    double u = hi ? s[2] : s[0], v = hi ? s[3] : s[1];
+    u += __shfl_xor_sync(0xffffffffu, hi ? s[0] : s[2], 16);
+    v += __shfl_xor_sync(0xffffffffu, hi ? s[1] : s[3], 16);
+    t = hi2 ? v : u;
+    t += __shfl_xor_sync(0xffffffffu, hi2 ? u : v, 8);
+    i += (hi ? 2 : 0) + (hi2 ? 1 : 0);
+  }
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  if ((lane & (R == 1 ? 31 : 7)) == 0 && i < n) d->x[i] = (T)t;
 }
 
 #define MGD_DISPATCH_FMT(K, fmt, maxrows, ny, s, descs)                                        \
@@ -426,8 +469,12 @@ void launch_phase(int phase, int fmtA, int fmtRP, const LDesc<T>* d_descs, int n
       break;
     case PH_JAC1: launch_k(k_jac1<T>, dim3(dim3(cdiv(maxrows, kVThreads), ndesc)), dim3(kVThreads), 0, s, d_descs); break;
     case PH_COARSE:
-      // one 1024-thread CTA per subsystem: a warp per row of the dense inverse
-      launch_k(k_coarse<T>, dim3(dim3(1, ndesc)), dim3(1024), sizeof(double) * maxrows, s, d_descs);
+      // four rows a warp once that still gives every SM two blocks
+      if ((long long)maxrows * ndesc >= 152 * 2 * 4 * (kDenseThreads / 32))
+        launch_k(k_coarse<T, 4>, dim3(cdiv(maxrows, 4 * (kDenseThreads / 32)), ndesc), dim3(kDenseThreads), 0, s,
+                 d_descs);
+      else
+        launch_k(k_coarse<T, 1>, dim3(cdiv(maxrows, kDenseThreads / 32), ndesc), dim3(kDenseThreads), 0, s, d_descs);
       break;
   }
   MGD_LAUNCH_CHECK();
@@ -680,6 +727,120 @@ __global__ void __launch_bounds__(kTailThreads) k_vtail(const TailSub<T>* __rest
     });
     cl.sync();
   }
+}
+
+// The cycle from a coarse level down is one linear map, and at a few hundred
+// rows its dense matrix costs less to apply than the levels' launches (three
+// per level at ~2.5 us in a graph; Gauss-Seidel: two per colour, ~60 colours).
+// This kernel forms it by running the cycle, phase by phase as the per-level
+// kernels do, on unit vectors: a block takes kCycCols of them (a lane each)
+// through all levels, its warps share the rows, and the work vectors hold the
+// block's columns side by side, so every access to them is coalesced.
+constexpr int kCycThreads = 512;
+
+__device__ __forceinline__ double cyc_row(const int* __restrict__ rp, const int* __restrict__ ci,
+                                          const double* __restrict__ v, const double* x, int r) {
+  double s = 0.0;
+  const int e = __ldg(rp + r + 1);
+#pragma unroll 4
+  for (int p = __ldg(rp + r); p < e; ++p) s += __ldg(v + p) * x[(size_t)__ldg(ci + p) * kCycCols];
+  return s;
+}
+
+__global__ void __launch_bounds__(kCycThreads) k_cycle_columns(const CycSub* __restrict__ subs,
+                                                               double* __restrict__ ws) {
+  int sub = 0;
+  while ((int)blockIdx.x >= subs[sub + 1].blk0) ++sub;
+  const CycSub S = subs[sub];
+  const int n0 = S.lev[0].n, cblk = (int)blockIdx.x - S.blk0, c0 = cblk * kCycCols;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int nw = kCycThreads / 32;
+  double* w = ws + S.ws0 + (size_t)cblk * (kCycCols * kCycVecs) * S.rows + lane;
+  // vector v (0 right-hand side, 1 iterate, 2 residual, then the output) of
+  // the level whose rows start at `base` within the chain
+  auto vec = [&](size_t base, int n, int v) { return w + (base * kCycVecs + (size_t)v * n) * kCycCols; };
+  auto at = [](int r) { return (size_t)r * kCycCols; };
+  size_t base = 0;
+  {
+    double* b = vec(0, n0, 0);
+    for (int r = warp; r < n0; r += nw) b[at(r)] = r == c0 + lane ? 1.0 : 0.0;
+  }
+  __syncthreads();
+  const int L = S.nlev;
+  auto sweep = [&](const LDesc<double>* d, const double* b, double* x, int sw) {
+    const int e = d->koff[sw + 1];
+    for (int q = d->koff[sw] + warp; q < e; q += nw) {
+      const int r = d->perm[q];
+      x[at(r)] += (b[at(r)] - cyc_row(d->rp, d->ci, d->v, x, r)) * d->gdinv[r];
+    }
+    __syncthreads();
+  };
+  for (int k = 0; k < L - 1; ++k) {
+    const LDesc<double>* d = S.lev + k;
+    const int n = d->n, nc = d->nc, nk = d->nk;
+    const double* b = vec(base, n, 0);
+    double *x = vec(base, n, 1), *res = vec(base, n, 2);
+    for (int r = warp; r < n; r += nw)
+      x[at(r)] = nk == 0 ? d->dinv[r] * b[at(r)] : d->key[r] == 0 ? b[at(r)] * d->gdinv[r] : 0.0;
+    __syncthreads();
+    for (int sw = 1; sw < nk; ++sw) sweep(d, b, x, sw);
+    for (int r = warp; r < n; r += nw) res[at(r)] = b[at(r)] - cyc_row(d->rp, d->ci, d->v, x, r);
+    __syncthreads();
+    base += n;
+    double* bc = vec(base, nc, 0);
+    for (int r = warp; r < nc; r += nw) bc[at(r)] = cyc_row(d->rrp, d->rci, d->rv, res, r);
+    __syncthreads();
+  }
+  const double* xc;  // the output of the level below
+  {
+    const LDesc<double>* d = S.lev + (L - 1);
+    const int n = d->n;
+    const double* b = vec(base, n, 0);
+    double *x = vec(base, n, 1), *res = vec(base, n, 2);
+    if (S.coarse_lu) {
+      for (int r = warp; r < n; r += nw) {
+        double s = 0.0;
+#pragma unroll 4
+        for (int j = 0; j < n; ++j) s += d->cinv[(size_t)r * n + j] * b[at(j)];
+        x[at(r)] = s;
+      }
+      xc = x;
+    } else {  // two l1-Jacobi sweeps from zero
+      for (int r = warp; r < n; r += nw) x[at(r)] = d->dinv[r] * b[at(r)];
+      __syncthreads();
+      for (int r = warp; r < n; r += nw)
+        res[at(r)] = x[at(r)] + d->dinv[r] * (b[at(r)] - cyc_row(d->rp, d->ci, d->v, x, r));
+      xc = res;
+    }
+  }
+  __syncthreads();
+  for (int k = L - 2; k >= 0; --k) {
+    const LDesc<double>* d = S.lev + k;
+    const int n = d->n, nk = d->nk;
+    base -= n;
+    const double* b = vec(base, n, 0);
+    double *x = vec(base, n, 1), *res = vec(base, n, 2);
+    for (int r = warp; r < n; r += nw) x[at(r)] += cyc_row(d->prp, d->pci, d->pv, xc, r);
+    __syncthreads();
+    for (int sw = nk - 1; sw >= 0; --sw) sweep(d, b, x, sw);
+    if (nk == 0) {
+      for (int r = warp; r < n; r += nw)
+        res[at(r)] = x[at(r)] + d->dinv[r] * (b[at(r)] - cyc_row(d->rp, d->ci, d->v, x, r));
+      __syncthreads();
+    }
+    xc = nk == 0 ? res : x;
+  }
+  if (c0 + lane >= n0) return;
+  for (int r = warp; r < n0; r += nw) {
+    S.out[(size_t)r * n0 + c0 + lane] = xc[at(r)];
+    if (S.outT) S.outT[(size_t)(c0 + lane) * n0 + r] = xc[at(r)];
+  }
+}
+
+void launch_cycle_columns(const CycSub* d_subs, int nblocks, double* ws, cudaStream_t s) {
+  if (nblocks <= 0) return;
+  k_cycle_columns<<<nblocks, kCycThreads, 0, s>>>(d_subs, ws);
+  MGD_LAUNCH_CHECK();
 }
 
 template <typename T>

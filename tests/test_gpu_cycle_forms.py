@@ -117,3 +117,65 @@ def test_gram_schmidt_grid_not_finite(gpu):
         assert e.value.code == 5
     x, it, rr, rc = slv.solve(torch.from_numpy(s.b))
     assert rc == 0 and rr <= 1e-8
+
+
+_DENSE = """
+import json, sys
+import torch
+sys.path.insert(0, sys.argv[1])
+from paper_2002_04958_gb300 import inputs, mgdamg
+out = []
+for G, dims, kind, prec, smoother, trans in json.loads(sys.argv[2]):
+    s = inputs.make_system(G, dims, multigroup=True)
+    slv = mgdamg.Solver(autotune=1, batched=1, use_graph=1, precision=prec, smoother=smoother,
+                        keep_transpose=trans, max_coarse=20).setup_system(s, kind)
+    b = torch.from_numpy(s.b)
+    lam = slv.solve_transpose(b)[0].cpu().tolist() if trans else []
+    out.append(dict(tail=[p["tail"] for p in slv.plan()], depth=[p["depth"] for p in slv.plan()],
+                    z=slv.precond_apply(b).cpu().tolist(), lam=lam))
+print(json.dumps(out))
+"""
+
+
+def test_dense_coarse_levels_match_oracle(gpu, orc, tmp_path):
+    # the levels from any one down as a dense matrix per subsystem (tail "level 1" in the tuning file), for both
+    # smoothers, a stalled coarsest level (20 groups) and the transposed cycle; the FP64 bounds are those of the
+    # other applies and transposed solves, FP32 as above
+    cases = [(2, (19, 17), "bd", 0, 0, 1), (2, (19, 17), "amg", 0, 1, 1), (20, (13, 11), "schur2", 0, 0, 0),
+             (20, (13, 11), "schur1", 0, 1, 0), (4, (23, 19), "bd", 1, 0, 0), (1, (40, 37), "amg", 0, 0, 1)]
+    path = tmp_path / "tune.txt"
+
+    def run():
+        p = subprocess.run([sys.executable, "-c", _DENSE, ROOT, json.dumps(cases)], capture_output=True, text=True,
+                           env=dict(os.environ, MGD_TUNE_CACHE=str(path)), timeout=600)
+        assert p.returncode == 0, p.stderr[-2000:]
+        return json.loads(p.stdout.strip().splitlines()[-1])
+
+    run()
+    lines = path.read_text().splitlines()
+    ref = []
+    for G, dims, kind, _, smoother, trans in cases:
+        s = inputs.make_system(G, dims, multigroup=True)
+        A = orc.csr_of_system(s)
+        M = orc.Block(A, s.G, s.N, kind, orc.opts(smoother=smoother, max_coarse=20))
+        ref.append((M.apply(s.b), orc.fgmres(A, s.b, M, tol=1e-8, transpose=True)[0] if trans else None))
+    seen = set()
+    for level in (1, 2, 3, 99):  # 99: no dense level
+        forced = []
+        for ln in lines:
+            fs = ln.split("|")
+            if len(fs[0].split()) > 3:
+                fs[5] = f"{level} 1"
+            forced.append("|".join(fs))
+        path.write_text("\n".join(forced) + "\n")
+        for case, r, (zo, lo) in zip(cases, run(), ref):
+            for t, d in zip(r["tail"], r["depth"]):
+                assert t == min(level, d), (level, case)
+                seen.add(t < d)
+            z = np.array(r["z"])
+            tol = 1e-12 if case[3] == 0 else 1e-4
+            assert np.linalg.norm(z - zo) <= tol * np.linalg.norm(zo), (level, case)
+            if lo is not None:
+                lam = np.array(r["lam"])
+                assert np.linalg.norm(lam - lo) <= 1e-10 * np.linalg.norm(lo), (level, case)
+    assert seen == {True, False}
