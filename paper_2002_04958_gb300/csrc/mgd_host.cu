@@ -313,66 +313,97 @@ static Csr transpose(Arena& a, const Csr& X, cudaStream_t s, Scratch* keep = nul
   return T;
 }
 
-// SELL-32 copy of A in the V-cycle's precision only (FP32 values when mixed,
-// else FP64); with dinv given, also A D^-1 in the same layout (vpre); the
-// values themselves only with `values` (levels with Q never read them).
-static Sell build_sell(Arena& a, const Csr& A, bool mixed, cudaStream_t s, const int* selfmap = nullptr,
-                       const double* dinv = nullptr, bool values = true) {
+static JointOff one_operator(int n) {
+  JointOff o;
+  o.n = 1;
+  o.off[1] = n;
+  return o;
+}
+
+// ceil(rows / per) units for each operator
+static JointOff units_of(const JointOff& rows, int per) {
+  JointOff u;
+  u.n = rows.n;
+  for (int k = 0; k < rows.n; ++k) u.off[k + 1] = u.off[k] + (rows.off[k + 1] - rows.off[k] + per - 1) / per;
+  return u;
+}
+
+// SELL-32 copy of A (operators at `rows`, columns made local) in the V-cycle's
+// precision only (FP32 values when mixed, else FP64); with dinv given, also
+// A D^-1 in the same layout (vpre); the values themselves only for the
+// operators of vmask (levels with Q never read them).
+static Sell build_sell(Arena& a, const Csr& A, const JointOff& rows, bool mixed, cudaStream_t s,
+                       const int* selfmap = nullptr, const double* dinv = nullptr, unsigned vmask = ~0u) {
   Scratch sc(s);
+  const JointOff slices = units_of(rows, 32);
   Sell S;
   S.n = A.n;
-  S.nslices = (A.n + 31) / 32;
+  S.nslices = slices.off[slices.n];
   int* w = sc.alloc<int>(S.nslices);
-  launch_sell_widths(A.n, A.rp, w, s);
+  launch_sell_widths(rows, slices, A.rp, w, s);
   S.sptr = a.alloc<int>(S.nslices + 1);
   exclusive_scan(w, S.sptr, S.nslices, s);
   S.nstored = read_int(S.sptr + S.nslices, s);
   S.ci = a.alloc<int>(S.nstored);
   if (mixed) {
-    if (values) S.v32 = a.alloc<float>(S.nstored);
+    if (vmask) S.v32 = a.alloc<float>(S.nstored);
     if (dinv) S.vpre32 = a.alloc<float>(S.nstored);
-    launch_sell_fill(A.n, A.rp, A.ci, A.v, dinv, S.sptr, S.ci, S.v32, S.vpre32, s, selfmap);
+    launch_sell_fill<float>(rows, slices, A.rp, A.ci, A.v, dinv, S.sptr, S.ci, S.v32, S.vpre32, vmask, s, selfmap);
   } else {
-    if (values) S.v = a.alloc<double>(S.nstored);
+    if (vmask) S.v = a.alloc<double>(S.nstored);
     if (dinv) S.vpre = a.alloc<double>(S.nstored);
-    launch_sell_fill(A.n, A.rp, A.ci, A.v, dinv, S.sptr, S.ci, S.v, S.vpre, s, selfmap);
+    launch_sell_fill<double>(rows, slices, A.rp, A.ci, A.v, dinv, S.sptr, S.ci, S.v, S.vpre, vmask, s, selfmap);
   }
   return S;
 }
-
-// The level's smoother diagonal D^-1 = 1 / sum_j |a_ij|
-static void build_dinv(Arena& a, Level& lv, bool mixed, cudaStream_t s) {
-  if (lv.dinv) return;
-  lv.dinv = a.alloc<double>(lv.A.n);
-  if (mixed) lv.dinv32 = a.alloc<float>(lv.A.n);
-  launch_l1_dinv(lv.A.n, lv.A.rp, lv.A.v, lv.dinv, s, lv.dinv32);
+static Sell build_sell(Arena& a, const Csr& A, bool mixed, cudaStream_t s, const int* selfmap = nullptr,
+                       const double* dinv = nullptr, unsigned vmask = ~0u) {
+  return build_sell(a, A, one_operator(A.n), mixed, s, selfmap, dinv, vmask);
 }
 
-// Q = P - D^-1 A P of a level from its A P (arena arrays, turned into Q in place)
-static void build_q(Arena& a, Level& lv, const Csr& AP, bool mixed, cudaStream_t s) {
+// The smoother diagonal D^-1 = 1 / sum_j |a_ij|
+static void build_dinv(Arena& a, const Csr& A, double*& dinv, float*& dinv32, bool mixed, cudaStream_t s) {
+  if (dinv) return;
+  dinv = a.alloc<double>(A.n);
+  if (mixed) dinv32 = a.alloc<float>(A.n);
+  launch_l1_dinv(A.n, A.rp, A.v, dinv, s, dinv32);
+}
+
+// Q = P - D^-1 A P from A P (arena arrays, turned into Q in place, its columns
+// made local to the operators): length-sorted SELL-32 and, when mixed, the FP32
+// CSR values
+struct QForm {
+  float* v32 = nullptr;
+  Sell sell;
+  unsigned char* perm = nullptr;
+};
+static QForm build_q(Arena& a, const Csr& AP, const Csr& P, const double* dinv, const JointOff& rows,
+                     const JointOff& cols, bool mixed, cudaStream_t s) {
   Scratch sc(s);
-  const int n = AP.n, nwin = (n + kQWin - 1) / kQWin;
-  Sell& S = lv.qsell;
-  lv.Q = AP;
-  S.n = n;
+  const JointOff wins = units_of(rows, kQWin);
+  const int nwin = wins.off[wins.n];
+  QForm q;
+  Sell& S = q.sell;
+  S.n = AP.n;
   S.nslices = nwin * (kQWin / 32);
-  lv.qperm = a.alloc<unsigned char>((size_t)nwin * kQWin);
+  q.perm = a.alloc<unsigned char>((size_t)nwin * kQWin);
   int* w = sc.alloc<int>(S.nslices);
-  launch_q_order(n, AP.rp, lv.qperm, w, s);
+  launch_q_order(rows, wins, AP.rp, q.perm, w, s);
   S.sptr = a.alloc<int>(S.nslices + 1);
   exclusive_scan(w, S.sptr, S.nslices, s);
   S.nstored = read_int(S.sptr + S.nslices, s);
   S.ci = a.alloc<int>(S.nstored);
   if (mixed) {
-    lv.qv32 = a.alloc<float>(AP.nnz);
+    q.v32 = a.alloc<float>(AP.nnz);
     S.v32 = a.alloc<float>(S.nstored);
-    launch_q_fill<float>(n, AP.rp, AP.ci, AP.v, lv.qv32, lv.P.rp, lv.P.ci, lv.P.v, lv.dinv, lv.qperm, S.sptr, S.ci,
+    launch_q_fill<float>(rows, cols, wins, AP.rp, AP.ci, AP.v, q.v32, P.rp, P.ci, P.v, dinv, q.perm, S.sptr, S.ci,
                          S.v32, s);
   } else {
     S.v = a.alloc<double>(S.nstored);
-    launch_q_fill<double>(n, AP.rp, AP.ci, AP.v, nullptr, lv.P.rp, lv.P.ci, lv.P.v, lv.dinv, lv.qperm, S.sptr, S.ci,
+    launch_q_fill<double>(rows, cols, wins, AP.rp, AP.ci, AP.v, nullptr, P.rp, P.ci, P.v, dinv, q.perm, S.sptr, S.ci,
                           S.v, s);
   }
+  return q;
 }
 
 static float* cast32(Arena& a, const double* x, int n, cudaStream_t s) {
@@ -444,15 +475,20 @@ static void gs_order(Arena& ar, Level& lv, int level, unsigned long long seed, c
 }
 
 // One coarsening pass on A (Section 3.1): strength, PMIS with the weight stream
-// 1000 + lid, interpolation.  CF and P come from `keep` when given (a pass
-// whose result is not kept as a level), else from the arena.  Returns false
-// when the pass stalls (no C point, or all C).
+// 1000 + lid, interpolation, for the operators of `active` among those at
+// `rows` (the others keep no point).  CF and P come from `keep` when given (a
+// pass whose result is not kept as a level), else from the arena.  An operator
+// stalls with no C point, or all C, and keeps none; returns false when every
+// one does.
 struct Pass {
   signed char* CF = nullptr;
   int nc = 0;
+  JointOff cols;          // the operators' coarse points
+  unsigned stalled = 0;   // active operators that keep none
   Csr P;
 };
-static bool coarsen_pass(SetupCtx& sc, const Csr& A, int lid, Scratch* keep, Pass& out) {
+static bool coarsen_pass(SetupCtx& sc, const Csr& A, const JointOff& rows, unsigned active, int lid, Scratch* keep,
+                         Pass& out) {
   Arena& ar = *sc.arena;
   cudaStream_t s = sc.s;
   const mgd_opts& o = *sc.o;
@@ -460,7 +496,7 @@ static bool coarsen_pass(SetupCtx& sc, const Csr& A, int lid, Scratch* keep, Pas
   Scratch tmp(s);
   PhaseTimer pt_str(sc.clk, SP_STRENGTH);
   uint8_t* S = tmp.alloc<uint8_t>(A.nnz);
-  launch_strength(n, A.rp, A.ci, A.v, o.theta_str, S, s);
+  launch_strength(n, A.rp, A.ci, A.v, o.theta_str, S, rows, active, s);
   int* cnt = tmp.alloc<int>(2 * (size_t)n);  // strong counts, then the fill cursors
   int* cur = cnt + n;
   MGD_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int) * 2 * (size_t)n, s));
@@ -473,7 +509,7 @@ static bool coarsen_pass(SetupCtx& sc, const Csr& A, int lid, Scratch* keep, Pas
   PhaseTimer pt_pmis(sc.clk, SP_PMIS);
   double* w = tmp.alloc<double>(n);
   signed char* CF = keep ? keep->alloc<signed char>(n) : ar.alloc<signed char>(n);
-  launch_pmis_init(n, A.rp, S, cnt, o.seed, lid, w, CF, s);
+  launch_pmis_init(n, A.rp, S, cnt, o.seed, lid, rows, w, CF, s);
   uint8_t* newc = tmp.alloc<uint8_t>(n);
   int* und = tmp.alloc<int>(1);
   // rounds are idempotent once every point is decided, so the undecided
@@ -487,23 +523,41 @@ static bool coarsen_pass(SetupCtx& sc, const Csr& A, int lid, Scratch* keep, Pas
   PhaseTimer pt_int(sc.clk, SP_INTERP);
   int* pcnt = tmp.alloc<int>(n);
   int* isc = tmp.alloc<int>(n);
-  launch_interp_count(n, A.rp, A.ci, S, CF, pcnt, isc, s);
   int* cidx = tmp.alloc<int>(n + 1);
-  exclusive_scan(isc, cidx, n, s);
+  int* dcols = tmp.alloc<int>(kMaxJoint + 1);
   // extended+i: upper bounds of the distance-two interpolatory sets, read
-  // back with the coarse count in one synchronisation
+  // back with the coarse counts in one synchronisation
   int* ub = nullptr;
   long long* off = nullptr;
   long long tot = 0;
-  if (o.interp_type == 1) {
-    ub = tmp.alloc<int>(n);
-    launch_exti_ub(n, A.rp, A.ci, S, CF, pcnt, ub, s);
-    off = tmp.alloc<long long>(n + 1);
-    launch_offsets64(ub, off, n, s);
-    MGD_CUDA(cudaMemcpyAsync(&tot, off + n, sizeof(long long), cudaMemcpyDeviceToHost, s));
+  JointOff cols;
+  for (bool again = true; again;) {
+    launch_interp_count(n, A.rp, A.ci, S, CF, pcnt, isc, s);
+    exclusive_scan(isc, cidx, n, s);
+    if (o.interp_type == 1) {
+      if (!ub) ub = tmp.alloc<int>(n);
+      launch_exti_ub(n, A.rp, A.ci, S, CF, pcnt, ub, s);
+      if (!off) off = tmp.alloc<long long>(n + 1);
+      launch_offsets64(ub, off, n, s);
+      MGD_CUDA(cudaMemcpyAsync(&tot, off + n, sizeof(long long), cudaMemcpyDeviceToHost, s));
+    }
+    launch_pick_ints(rows, cidx, dcols, s);
+    cols.n = rows.n;
+    MGD_CUDA(cudaMemcpyAsync(cols.off, dcols, sizeof(int) * (rows.n + 1), cudaMemcpyDeviceToHost, s));
+    MGD_CUDA(cudaStreamSynchronize(s));
+    again = false;
+    for (int k = 0; k < rows.n; ++k) {
+      const int nk = rows.off[k + 1] - rows.off[k], ck = cols.off[k + 1] - cols.off[k];
+      if (!(active >> k & 1u)) continue;
+      if (ck == 0) out.stalled |= 1u << k;
+      if (ck > 0 && ck == nk) {  // all C: this operator is not coarsened
+        MGD_CUDA(cudaMemsetAsync(CF + rows.off[k], 0xff, nk, s));
+        again = true;
+      }
+    }
   }
-  int nc = read_int(cidx + n, s);
-  if (nc == 0 || nc == n) return false;
+  const int nc = cols.off[cols.n];
+  if (nc == 0) return false;
   Csr P;
   P.n = n;
   P.m = nc;
@@ -535,6 +589,7 @@ static bool coarsen_pass(SetupCtx& sc, const Csr& A, int lid, Scratch* keep, Pas
   pt_int.stop();
   out.CF = CF;
   out.nc = nc;
+  out.cols = cols;
   out.P = P;
   return true;
 }
@@ -553,7 +608,7 @@ static void aggressive_pass(SetupCtx& sc, const Csr& A, int l, Pass& pass) {
   Csr AP1 = spgemm(ar, A, pass.P, s, &ak);
   Csr A1 = spgemm(ar, R1, AP1, s, &ak);
   Pass p2;
-  if (!coarsen_pass(sc, A1, 100 + l, &ak, p2)) return;
+  if (!coarsen_pass(sc, A1, one_operator(A1.n), 1u, 100 + l, &ak, p2)) return;
   Csr P = spgemm(ar, pass.P, p2.P, s);
   int* flag = ak.alloc<int>(n);
   int* cidx = ak.alloc<int>(n + 1);
@@ -565,9 +620,45 @@ static void aggressive_pass(SetupCtx& sc, const Csr& A, int l, Pass& pass) {
   MGD_CUDA(cudaStreamSynchronize(s));
 }
 
+// Inverses of the coarsest levels with at most max_coarse rows (local columns)
+static void coarse_inverses(Arena& ar, const std::vector<Hier*>& hs, int max_coarse, cudaStream_t s) {
+  Scratch tmp(s);
+  int* st = tmp.alloc<int>(1);
+  MGD_CUDA(cudaMemsetAsync(st, 0, sizeof(int), s));
+  std::vector<InvDesc> small;
+  int maxn = 0, any = 0;
+  for (Hier* h : hs) {
+    const Csr& A = h->L.back().A;
+    const int n = A.n;
+    if (n > max_coarse) continue;
+    h->coarse_lu = true;
+    h->cn = n;
+    h->cinv = ar.alloc<double>((size_t)n * n);
+    h->cinvT = ar.alloc<double>((size_t)n * n);
+    any = 1;
+    if (n <= kGjMax) {
+      small.push_back(InvDesc{n, A.rp, A.ci, A.v, h->cinv, h->cinvT});
+      maxn = std::max(maxn, n);
+      continue;
+    }
+    double* a = tmp.alloc<double>((size_t)n * n);
+    int* piv = tmp.alloc<int>(n);
+    launch_densify(n, A.rp, A.ci, A.v, a, s);
+    launch_dense_inverse(n, a, piv, h->cinv, h->cinvT, st, s);
+  }
+  if (!any) return;
+  if (!small.empty()) {
+    InvDesc* d = tmp.alloc<InvDesc>(small.size());
+    MGD_CUDA(cudaMemcpyAsync(d, small.data(), sizeof(InvDesc) * small.size(), cudaMemcpyHostToDevice, s));
+    launch_dense_inverses(d, (int)small.size(), maxn, st, s);
+  }
+  if (read_int(st, s) != 0) throw Error{MGD_ESINGULAR, "zero pivot in the coarsest-level elimination"};
+}
+
 // Section 3.1 setup: strength -> PMIS -> interpolation -> R = P^T -> A_c = R (A P),
 // level by level until the coarsest criterion; then smoother diagonals,
-// kernel layouts, FP32 copies and the coarsest dense inverse.
+// kernel layouts, FP32 copies and the coarsest dense inverse.  One operator;
+// for Gauss-Seidel and aggressive coarsening (others: build_joint).
 static void build_hierarchy(SetupCtx& sc, Hier& h, const Csr& A0) {
   Arena& ar = *sc.arena;
   cudaStream_t s = sc.s;
@@ -580,7 +671,7 @@ static void build_hierarchy(SetupCtx& sc, Hier& h, const Csr& A0) {
     int n = lv.A.n;
     if (n <= o.max_coarse || l == o.max_levels - 1) break;
     Pass pass;
-    if (!coarsen_pass(sc, lv.A, l, nullptr, pass)) break;  // coarsening stalled: this level is the coarsest
+    if (!coarsen_pass(sc, lv.A, one_operator(n), 1u, l, nullptr, pass)) break;  // coarsening stalled: this level is the coarsest
     if (l < o.agg_levels) aggressive_pass(sc, lv.A, l, pass);
     lv.CF = pass.CF;
     lv.nc = pass.nc;
@@ -603,8 +694,12 @@ static void build_hierarchy(SetupCtx& sc, Hier& h, const Csr& A0) {
     pt_rap.stop();
     if (with_q) {
       PhaseTimer pt_q(sc.clk, SP_FINALIZE);
-      build_dinv(ar, lv, sc.mixed, s);
-      build_q(ar, lv, AP, sc.mixed, s);
+      build_dinv(ar, lv.A, lv.dinv, lv.dinv32, sc.mixed, s);
+      QForm q = build_q(ar, AP, P, lv.dinv, one_operator(n), one_operator(lv.nc), sc.mixed, s);
+      lv.Q = AP;
+      lv.qv32 = q.v32;
+      lv.qsell = q.sell;
+      lv.qperm = q.perm;
     }
     h.L.emplace_back();
     h.L.back().A = Ac;
@@ -614,7 +709,7 @@ static void build_hierarchy(SetupCtx& sc, Hier& h, const Csr& A0) {
   for (int l = 0; l < h.nlev(); ++l) {
     Level& lv = h.L[l];
     int n = lv.A.n;
-    build_dinv(ar, lv, sc.mixed, s);
+    build_dinv(ar, lv.A, lv.dinv, lv.dinv32, sc.mixed, s);
     if (lv.nk > 0) {
       lv.gdinv = ar.alloc<double>(n);
       launch_diag_inv(n, lv.A.rp, lv.A.ci, lv.A.v, lv.gdinv, s);
@@ -639,7 +734,7 @@ static void build_hierarchy(SetupCtx& sc, Hier& h, const Csr& A0) {
     // value (or the FP64 product a_ij d_j) rounded once.
     const bool jac = lv.nk == 0;
     const double* pre = jac ? lv.dinv : nullptr;
-    lv.sell = build_sell(ar, lv.A, sc.mixed, s, nullptr, pre, lv.qperm == nullptr);
+    lv.sell = build_sell(ar, lv.A, sc.mixed, s, nullptr, pre, lv.qperm ? 0u : ~0u);
     if (sc.mixed) {
       lv.v32 = ar.alloc<float>(lv.A.nnz);
       if (jac) lv.vpre32 = ar.alloc<float>(lv.A.nnz);
@@ -679,22 +774,217 @@ static void build_hierarchy(SetupCtx& sc, Hier& h, const Csr& A0) {
   MGD_CUDA(cudaStreamSynchronize(s));
   pt_fin.stop();
   PhaseTimer pt_co(sc.clk, SP_COARSE);
-  Level& last = h.L.back();
-  if (last.A.n <= o.max_coarse) {
-    int n = last.A.n;
-    Scratch tmp(s);
-    double* a = tmp.alloc<double>((size_t)n * n);
-    int* piv = tmp.alloc<int>(n);
-    int* st = tmp.alloc<int>(1);
-    MGD_CUDA(cudaMemsetAsync(st, 0, sizeof(int), s));
-    h.cinv = ar.alloc<double>((size_t)n * n);
-    h.cinvT = ar.alloc<double>((size_t)n * n);
-    launch_densify(n, last.A.rp, last.A.ci, last.A.v, a, s);
-    launch_dense_inverse(n, a, piv, h.cinv, h.cinvT, st, s);
-    if (read_int(st, s) != 0) throw Error{MGD_ESINGULAR, "zero pivot in the coarsest-level elimination"};
-    h.coarse_lu = true;
-    h.cn = n;
+  coarse_inverses(ar, {&h}, o.max_coarse, s);
+}
+
+// The same for several operators at once, l1-Jacobi levels: they are set up as
+// one block-diagonal matrix, level by level, so that a step of the setup is one
+// launch for all of them (22 operators on 16 threads and streams made some
+// 10,000 launches, and what the threads shared was the driver).  Every row is
+// treated as it would be alone -- the same sums in the same order, the weights
+// of its index within its operator, the same coarsest criterion -- so the
+// hierarchies are the same bit for bit.  An operator that is done keeps no
+// coarse point and leaves the joint matrix with the next level.  At the end the
+// operators' levels are views of the joint arrays, their columns made local.
+static void build_joint(SetupCtx& sc, const std::vector<Hier*>& hs, const std::vector<const Csr*>& A0) {
+  Arena& ar = *sc.arena;
+  cudaStream_t s = sc.s;
+  const mgd_opts& o = *sc.o;
+  const int nops = (int)hs.size();
+  struct JLevel {
+    Csr A, P, R, AT, Q;
+    JointOff rows;
+    unsigned coarsest = 0;  // operators that end here
+    signed char* CF = nullptr;
+    double* dinv = nullptr;
+    float* dinv32 = nullptr;
+    QForm q;
+  };
+  std::vector<JLevel> L(1);
+  Scratch first(s, ar.pool);  // the joint level 0 (the operators keep their own arrays there)
+  std::vector<int> entry0(nops + 1, 0);
+  L[0].rows.n = nops;
+  for (int k = 0; k < nops; ++k) {
+    L[0].rows.off[k + 1] = L[0].rows.off[k] + A0[k]->n;
+    entry0[k + 1] = entry0[k] + A0[k]->nnz;
   }
+  if (nops == 1) {
+    L[0].A = *A0[0];
+  } else {
+    Csr J;
+    J.n = J.m = L[0].rows.off[nops];
+    J.nnz = entry0[nops];
+    J.rp = first.alloc<int>(J.n + 1);
+    J.ci = first.alloc<int>(J.nnz);
+    J.v = first.alloc<double>(J.nnz);
+    for (int k = 0; k < nops; ++k)
+      launch_join(A0[k]->n, A0[k]->rp, A0[k]->ci, A0[k]->v, L[0].rows.off[k], entry0[k], J.rp, J.ci, J.v, s);
+    L[0].A = J;
+  }
+  for (int l = 0;; ++l) {
+    unsigned act = 0;
+    for (int k = 0; k < nops; ++k) {
+      const int nk = L[l].rows.off[k + 1] - L[l].rows.off[k];
+      if (nk == 0 && l > 0) continue;
+      if (nk <= o.max_coarse || l == o.max_levels - 1) L[l].coarsest |= 1u << k;
+      else act |= 1u << k;
+    }
+    if (!act) break;
+    Pass pass;
+    const bool more = coarsen_pass(sc, L[l].A, L[l].rows, act, l, nullptr, pass);
+    L[l].coarsest |= pass.stalled;
+    if (!more) break;
+    L.emplace_back();
+    JLevel& lv = L[l];
+    JLevel& nx = L[l + 1];
+    nx.rows = pass.cols;
+    lv.CF = pass.CF;
+    lv.P = pass.P;
+    PhaseTimer pt_tr(sc.clk, SP_TRANSPOSE);
+    lv.R = transpose(ar, lv.P, s);
+    pt_tr.stop();
+    PhaseTimer pt_ap(sc.clk, SP_AP);
+    lv.Q = spgemm(ar, lv.A, lv.P, s);
+    pt_ap.stop();
+    PhaseTimer pt_rap(sc.clk, SP_RAP);
+    nx.A = spgemm(ar, lv.R, lv.Q, s);
+    pt_rap.stop();
+    PhaseTimer pt_q(sc.clk, SP_FINALIZE);
+    build_dinv(ar, lv.A, lv.dinv, lv.dinv32, sc.mixed, s);
+    lv.q = build_q(ar, lv.Q, lv.P, lv.dinv, lv.rows, nx.rows, sc.mixed, s);
+  }
+  PhaseTimer pt_fin(sc.clk, SP_FINALIZE);
+  const int nlev = (int)L.size();
+  for (Hier* h : hs) h->L.clear();
+  for (int l = 0; l < nlev; ++l) {
+    JLevel& lv = L[l];
+    const bool down = l + 1 < nlev;
+    build_dinv(ar, lv.A, lv.dinv, lv.dinv32, sc.mixed, s);
+    // stalled coarsest levels are smoothed with the values themselves, the others (above a coarser one) with Q
+    unsigned vmask = 0;
+    for (int k = 0; k < nops; ++k)
+      if ((lv.coarsest >> k & 1u) && lv.rows.off[k + 1] - lv.rows.off[k] > o.max_coarse) vmask |= 1u << k;
+    Sell sell = build_sell(ar, lv.A, lv.rows, sc.mixed, s, nullptr, lv.dinv, vmask), sellT;
+    float *v32 = nullptr, *vpre32 = nullptr, *pv32 = nullptr, *rv32 = nullptr, *atv32 = nullptr, *atvpre32 = nullptr;
+    double *vpre = nullptr, *atvpre = nullptr;
+    if (sc.mixed) {
+      v32 = ar.alloc<float>(lv.A.nnz);
+      vpre32 = ar.alloc<float>(lv.A.nnz);
+      launch_colscale_f32(lv.A.nnz, lv.A.ci, lv.A.v, lv.dinv, v32, vpre32, s);
+      if (down) {
+        pv32 = cast32(ar, lv.P.v, lv.P.nnz, s);
+        rv32 = cast32(ar, lv.R.v, lv.R.nnz, s);
+      }
+    } else {
+      vpre = ar.alloc<double>(lv.A.nnz);
+      launch_colscale(lv.A.nnz, lv.A.ci, lv.A.v, lv.dinv, vpre, s);
+    }
+    if (sc.keepT) {
+      lv.AT = transpose(ar, lv.A, s);
+      sellT = build_sell(ar, lv.AT, lv.rows, sc.mixed, s, nullptr, lv.dinv);
+      if (sc.mixed) {
+        atv32 = ar.alloc<float>(lv.AT.nnz);
+        atvpre32 = ar.alloc<float>(lv.AT.nnz);
+        launch_colscale_f32(lv.AT.nnz, lv.AT.ci, lv.AT.v, lv.dinv, atv32, atvpre32, s);
+      } else {
+        atvpre = ar.alloc<double>(lv.AT.nnz);
+        launch_colscale(lv.AT.nnz, lv.AT.ci, lv.AT.v, lv.dinv, atvpre, s);
+      }
+      launch_localise(lv.rows, lv.rows, lv.AT.rp, lv.AT.ci, s);
+    }
+    if (l > 0) launch_localise(lv.rows, lv.rows, lv.A.rp, lv.A.ci, s);
+    if (down) {
+      launch_localise(lv.rows, L[l + 1].rows, lv.P.rp, lv.P.ci, s);
+      launch_localise(L[l + 1].rows, lv.rows, lv.R.rp, lv.R.ci, s);
+    }
+    // the operators' vectors b, xt, x, r in one zeroed block, each 256-byte aligned
+    const size_t es = sc.mixed ? sizeof(float) : sizeof(double);
+    auto pad = [&](int n) { return (es * n + 255) & ~(size_t)255; };
+    size_t bytes = 0;
+    for (int k = 0; k < nops; ++k) bytes += 4 * pad(lv.rows.off[k + 1] - lv.rows.off[k]);
+    char* vec = ar.alloc<char>(bytes);
+    MGD_CUDA(cudaMemsetAsync(vec, 0, bytes, s));
+    const JointOff slices = units_of(lv.rows, 32), wins = units_of(lv.rows, kQWin);
+    for (int k = 0; k < nops; ++k) {
+      const int r0 = lv.rows.off[k], n = lv.rows.off[k + 1] - r0;
+      if (n == 0 && l > 0) continue;
+      hs[k]->L.emplace_back();
+      Level& t = hs[k]->L.back();
+      // the joint arrays' entries of operator k start at row r0's; at level 0 the operator's own arrays start at 0
+      const size_t e0 = l == 0 ? entry0[k] : 0;
+      auto at = [](auto* p, size_t o) { return p ? p + o : p; };
+      auto view = [&](const Csr& J, int row, int nr, int m) {
+        Csr c = J;
+        c.rp = J.rp + row;
+        c.n = nr;
+        c.m = m;
+        return c;
+      };
+      t.A = l == 0 ? *A0[k] : view(lv.A, r0, n, n);
+      t.v32 = at(v32, e0);
+      t.vpre = at(vpre, e0);
+      t.vpre32 = at(vpre32, e0);
+      t.sell = sell;
+      t.sell.n = n;
+      t.sell.sptr = sell.sptr + slices.off[k];
+      t.dinv = lv.dinv + r0;
+      t.dinv32 = at(lv.dinv32, r0);
+      if (sc.keepT) {
+        t.AT = view(lv.AT, r0, n, n);
+        t.atv32 = atv32;
+        t.atvpre = atvpre;
+        t.atvpre32 = atvpre32;
+        t.sellT = sellT;
+        t.sellT.n = n;
+        t.sellT.sptr = sellT.sptr + slices.off[k];
+      }
+      if (!(lv.coarsest >> k & 1u)) {
+        const int c0 = L[l + 1].rows.off[k], nc = L[l + 1].rows.off[k + 1] - c0;
+        t.CF = lv.CF + r0;
+        t.nc = nc;
+        t.P = view(lv.P, r0, n, nc);
+        t.R = view(lv.R, c0, nc, n);
+        t.Q = view(lv.Q, r0, n, nc);
+        t.pv32 = pv32;
+        t.rv32 = rv32;
+        t.qv32 = lv.q.v32;
+        t.qsell = lv.q.sell;
+        t.qsell.n = n;
+        t.qsell.sptr = lv.q.sell.sptr + wins.off[k] * (kQWin / 32);
+        t.qperm = lv.q.perm + (size_t)wins.off[k] * kQWin;
+      }
+      t.b = vec;
+      t.xt = vec + pad(n);
+      t.x = vec + 2 * pad(n);
+      t.r = vec + 3 * pad(n);
+      vec += 4 * pad(n);
+    }
+  }
+  // every view's entry count: the difference of its first and last row pointers
+  if (nops > 1) {
+    std::vector<const int*> ends;
+    std::vector<Csr*> views;
+    for (Hier* h : hs)
+      for (Level& t : h->L)
+        for (Csr* v : {&t.A, &t.AT, &t.P, &t.R, &t.Q})
+          if (v->rp) {
+            views.push_back(v);
+            ends.push_back(v->rp);
+            ends.push_back(v->rp + v->n);
+          }
+    Scratch tmp(s);
+    const int** d = tmp.alloc<const int*>(ends.size());
+    int* dv = tmp.alloc<int>(ends.size());
+    std::vector<int> got(ends.size());
+    MGD_CUDA(cudaMemcpyAsync(d, ends.data(), sizeof(int*) * ends.size(), cudaMemcpyHostToDevice, s));
+    launch_gather_ints(d, (int)ends.size(), dv, s);
+    MGD_CUDA(cudaMemcpyAsync(got.data(), dv, sizeof(int) * got.size(), cudaMemcpyDeviceToHost, s));
+    MGD_CUDA(cudaStreamSynchronize(s));
+    for (size_t i = 0; i < views.size(); ++i) views[i]->nnz = got[2 * i + 1] - got[2 * i];
+  }
+  pt_fin.stop();
+  PhaseTimer pt_co(sc.clk, SP_COARSE);
+  coarse_inverses(ar, hs, o.max_coarse, s);
 }
 
 // ------------------------------------------------------------------ batched V-cycle plans
@@ -1466,8 +1756,10 @@ static void finalize_op(mgd_ctx* c, InvOp& op, cudaStream_t st) {
     op.b = c->ar.alloc<char>(es * op.n, true, st);
     op.x = c->ar.alloc<char>(es * op.n, true, st);
   } else {
-    SetupCtx sc{&c->ar, st, &c->o, mixed(c), c->o.keep_transpose != 0, &c->phases};
-    build_hierarchy(sc, op.h, op.A);
+    if (op.h.L.empty()) {
+      SetupCtx sc{&c->ar, st, &c->o, mixed(c), c->o.keep_transpose != 0, &c->phases};
+      build_hierarchy(sc, op.h, op.A);
+    }
     op.b = op.h.L[0].b;
     op.x = op.h.L[0].x;
   }
@@ -1496,6 +1788,35 @@ static void finalize_op(mgd_ctx* c, InvOp& op, cudaStream_t st) {
 #define MGD_SETUP_OVERSUB 1
 #endif
 
+// The hierarchies of operators [first, last) that take l1-Jacobi V-cycles,
+// jointly, in groups whose level-0 entries stay well inside 32-bit indices
+static void build_joint_ops(mgd_ctx* c, size_t first, size_t last) {
+  SetupCtx sc{&c->ar, c->s, &c->o, mixed(c), c->o.keep_transpose != 0, &c->phases};
+  struct Region {  // setup scratch of the context stream
+    ScratchRegion r;
+    explicit Region(mgd_ctx* c) : r(c->s, c->ar.pool) { tl_region = &r; }
+    ~Region() { tl_region = nullptr; }
+  } region(c);
+  std::vector<Hier*> hs;
+  std::vector<const Csr*> as;
+  long long nnz = 0;
+  auto flush = [&] {
+    if (!hs.empty()) build_joint(sc, hs, as);
+    hs.clear();
+    as.clear();
+    nnz = 0;
+  };
+  for (size_t k = first; k < last; ++k) {
+    InvOp& op = c->ops[k];
+    if (op.jacobi) continue;
+    if (nnz + op.A.nnz > (1LL << 29) || (int)hs.size() == kMaxJoint) flush();
+    hs.push_back(&op.h);
+    as.push_back(&op.A);
+    nnz += op.A.nnz;
+  }
+  flush();
+}
+
 // Setup of independent operators runs concurrently: each worker thread owns a
 // CUDA stream and builds whole hierarchies, so the many small host round
 // trips of one hierarchy (scan totals, PMIS rounds) overlap with the others.
@@ -1504,6 +1825,11 @@ static void finalize_ops_parallel(mgd_ctx* c, size_t first, size_t last) {
   size_t nops = last - first;
   if (nops == 0) return;
   MGD_CUDA(cudaStreamSynchronize(c->s));
+  if (c->o.smoother == 0 && c->o.agg_levels == 0) {
+    build_joint_ops(c, first, last);
+    for (size_t k = first; k < last; ++k) finalize_op<T>(c, c->ops[k], c->s);
+    return;
+  }
   unsigned hw = std::thread::hardware_concurrency();
   size_t nthreads = std::min<size_t>(
       nops, std::max<unsigned>(1u, std::min<unsigned>((hw ? hw : 4) * MGD_SETUP_OVERSUB, MGD_SETUP_THREADS)));
@@ -3369,14 +3695,20 @@ int mgd_level_export(mgd_ctx* c, int op, int level, int* h_rp, int* h_ci, double
     auto cp = [&](void* dst, const void* src, size_t bytes) {
       if (dst && src && bytes) MGD_CUDA(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, c->s));
     };
-    cp(h_rp, lv.A.rp, sizeof(int) * (lv.A.n + 1));
-    cp(h_ci, lv.A.ci, sizeof(int) * lv.A.nnz);
-    cp(h_v, lv.A.v, sizeof(double) * lv.A.nnz);
+    // a level may be a view of joint arrays: its entries start at its first row pointer
+    auto csr = [&](const Csr& m, int* rp, int* ci, double* v) {
+      const int e0 = read_int(m.rp, c->s);
+      cp(rp, m.rp, sizeof(int) * (m.n + 1));
+      cp(ci, m.ci + e0, sizeof(int) * m.nnz);
+      cp(v, m.v + e0, sizeof(double) * m.nnz);
+      MGD_CUDA(cudaStreamSynchronize(c->s));
+      if (rp)
+        for (int i = 0; i <= m.n; ++i) rp[i] -= e0;
+    };
+    csr(lv.A, h_rp, h_ci, h_v);
     if (!last) {
       cp(h_cf, lv.CF, lv.A.n);
-      cp(h_prp, lv.P.rp, sizeof(int) * (lv.A.n + 1));
-      cp(h_pci, lv.P.ci, sizeof(int) * lv.P.nnz);
-      cp(h_pv, lv.P.v, sizeof(double) * lv.P.nnz);
+      csr(lv.P, h_prp, h_pci, h_pv);
     }
     MGD_CUDA(cudaStreamSynchronize(c->s));
     return MGD_OK;

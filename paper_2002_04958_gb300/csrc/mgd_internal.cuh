@@ -278,6 +278,15 @@ struct Csr {  // device CSR, FP64 values
   double* v = nullptr;
 };
 
+// Several operators set up as one block-diagonal matrix: row (or slice, or
+// window) offsets of the operators in the joint numbering.  Passed to kernels
+// by value.
+constexpr int kMaxJoint = 32;
+struct JointOff {
+  int n = 0;                    // operators
+  int off[kMaxJoint + 1] = {0};
+};
+
 // sparse-kernel formats chosen per level by the autotuner
 enum Fmt { FMT_SELL = 0, FMT_CSR1 = 1, FMT_CSR2 = 2, FMT_CSR4 = 3, FMT_CSR8 = 4, FMT_CSR16 = 5, FMT_CSR32 = 6,
            FMT_SELL2 = 7, FMT_SELL4 = 8,     // SELL-32 with each thread on the same lane of 2 / 4 adjacent
@@ -477,13 +486,15 @@ void launch_gamma_wd(int n, const int* rp, const int* ci, const double* v, doubl
                      cudaStream_t s);
 void launch_gamma_wc(int n, const double* d, const double* diag, double theta, int* count, cudaStream_t s);
 
+// rows: the operators' rows of a joint matrix; active: bit k set: operator k is coarsened (the others get no strong
+// connection)
 void launch_strength(int n, const int* rp, const int* ci, const double* v, double theta, uint8_t* S,
-                     cudaStream_t s);
+                     const JointOff& rows, unsigned active, cudaStream_t s);
 void launch_count_st(int n, const int* rp, const int* ci, const uint8_t* S, int* cnt, cudaStream_t s);
 void launch_fill_st(int n, const int* rp, const int* ci, const uint8_t* S, const int* strp, int* cursor,
                     int* stci, cudaStream_t s);
 void launch_pmis_init(int n, const int* rp, const uint8_t* S, const int* cnt, unsigned long long seed, int level,
-                      double* w, signed char* CF, cudaStream_t s);
+                      const JointOff& rows, double* w, signed char* CF, cudaStream_t s);
 void launch_pmis_round(int n, const int* rp, const int* ci, const uint8_t* S, const int* strp, const int* stci,
                        const double* w, signed char* CF, uint8_t* newc, int* undecided, cudaStream_t s);
 void launch_colour_init(int n, unsigned long long seed, int level, double* w, int* col, cudaStream_t s);
@@ -531,20 +542,43 @@ void launch_pctl_ac_count(int N, int nc, const int* const* brp, const int* const
 void launch_pctl_ac_fill(int N, int nc, int G, const int* const* brp, const int* const* bci,
                          const double* const* bv, const double* const* p, const double* const* dtab,
                          const int* acrp, int* acci, double* acv, cudaStream_t s);
-void launch_sell_widths(int n, const int* rp, int* w, cudaStream_t s);
-// SELL-32 copy of a CSR matrix; with d given, svpre gets A D^-1 in the same pass
-void launch_sell_fill(int n, const int* rp, const int* ci, const double* v, const double* d, const int* sptr,
-                      int* sci, double* sv, double* svpre, cudaStream_t s, const int* selfmap = nullptr);
-void launch_sell_fill(int n, const int* rp, const int* ci, const double* v, const double* d, const int* sptr,
-                      int* sci, float* sv, float* svpre, cudaStream_t s, const int* selfmap = nullptr);
+// joint SELL-32: slices of 32 rows that do not cross operators (slices: their offsets)
+void launch_sell_widths(const JointOff& rows, const JointOff& slices, const int* rp, int* w, cudaStream_t s);
+// SELL-32 copy of a CSR matrix with each operator's columns counted from its cols offset; with d given, svpre gets
+// A D^-1 in the same pass; values only for the operators of vmask; selfmap: padding column of a row (one operator)
+template <typename T>
+void launch_sell_fill(const JointOff& rows, const JointOff& slices, const int* rp, const int* ci, const double* v,
+                      const double* d, const int* sptr, int* sci, T* sv, T* svpre, unsigned vmask, cudaStream_t s,
+                      const int* selfmap = nullptr);
+// columns of a joint matrix (rows of operator k, columns from cols.off[k]) made local to each operator
+void launch_localise(const JointOff& rows, const JointOff& cols, const int* rp, int* ci, cudaStream_t s);
+// an operator's rows and entries into the joint level-0 matrix
+void launch_join(int n, const int* rp, const int* ci, const double* v, int row0, int entry0, int* jrp, int* jci,
+                 double* jv, cudaStream_t s);
+// out[k] = src[at.off[k]], k <= at.n
+void launch_pick_ints(const JointOff& at, const int* src, int* out, cudaStream_t s);
+// out[i] = *src[i]
+void launch_gather_ints(const int* const* src, int m, int* out, cudaStream_t s);
+// inverses (and their transposes) of several small matrices given in CSR with local columns
+struct InvDesc {
+  int n;
+  const int* rp;
+  const int* ci;
+  const double* v;
+  double* inv;
+  double* invT;
+};
+constexpr int kGjMax = 112;  // rows served by this kernel
+void launch_dense_inverses(const InvDesc* d, int nd, int maxn, int* status, cudaStream_t s);
 // Q = P - D^-1 A P (see k_q_fill): the window order and the slice widths, then
 // the values (q holds A P on entry, Q on return; q32: its FP32 copy, or nullptr)
 constexpr int kQWin = 256;  // rows per window
-void launch_q_order(int n, const int* rp, unsigned char* perm, int* widths, cudaStream_t s);
+void launch_q_order(const JointOff& rows, const JointOff& wins, const int* rp, unsigned char* perm, int* widths,
+                    cudaStream_t s);
 template <typename T>
-void launch_q_fill(int n, const int* rp, const int* ci, double* q, float* q32, const int* prp, const int* pci,
-                   const double* pv, const double* dinv, const unsigned char* perm, const int* sptr, int* sci, T* sv,
-                   cudaStream_t s);
+void launch_q_fill(const JointOff& rows, const JointOff& cols, const JointOff& wins, const int* rp, int* ci, double* q,
+                   float* q32, const int* prp, const int* pci, const double* pv, const double* dinv,
+                   const unsigned char* perm, const int* sptr, int* sci, T* sv, cudaStream_t s);
 void launch_colscale(long long nnz, const int* ci, const double* v, const double* d, double* out, cudaStream_t s);
 // FP32 values (vout) and FP32 A D^-1 (out, when d is given) of FP64 CSR values, one pass
 void launch_colscale_f32(long long nnz, const int* ci, const double* v, const double* d, float* vout, float* out,

@@ -11,6 +11,17 @@
 
 namespace mgd {
 
+// the operator of a joint matrix that holds row (slice, window) i
+__device__ __forceinline__ int joint_of(const JointOff& o, int i) {
+  int lo = 0, hi = o.n - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (o.off[mid] <= i) lo = mid;
+    else hi = mid - 1;
+  }
+  return lo;
+}
+
 // ------------------------------------------------------------------ scan
 // per block of kThreads * 4 outputs: exclusive sums of in[0..n_in) followed
 // by zeros (n outputs), and the block's total in bsum
@@ -312,9 +323,14 @@ void launch_gamma_wc(int n, const double* d, const double* diag, double theta, i
 }
 
 // ------------------------------------------------------------------ strength of connection (Section 3.1)
-__global__ void k_strength(int n, const int* rp, const int* ci, const double* v, double theta, uint8_t* S) {
+__global__ void k_strength(int n, const int* rp, const int* ci, const double* v, double theta, uint8_t* S,
+                           JointOff rows, unsigned active) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
+  if (!(active >> joint_of(rows, i) & 1u)) {
+    for (int p = rp[i]; p < rp[i + 1]; ++p) S[p] = 0;
+    return;
+  }
   double mx = 0.0;
   for (int p = rp[i]; p < rp[i + 1]; ++p)
     if (ci[p] != i && -v[p] > mx) mx = -v[p];
@@ -323,8 +339,8 @@ __global__ void k_strength(int n, const int* rp, const int* ci, const double* v,
 }
 
 void launch_strength(int n, const int* rp, const int* ci, const double* v, double theta, uint8_t* S,
-                     cudaStream_t s) {
-  k_strength<<<cdiv(n, kThreads), kThreads, 0, s>>>(n, rp, ci, v, theta, S);
+                     const JointOff& rows, unsigned active, cudaStream_t s) {
+  k_strength<<<cdiv(n, kThreads), kThreads, 0, s>>>(n, rp, ci, v, theta, S, rows, active);
   MGD_LAUNCH_CHECK();
 }
 
@@ -374,10 +390,10 @@ void launch_fill_st(int n, const int* rp, const int* ci, const uint8_t* S, const
 
 // weights w_i = |S^T_i| + u_i; isolated points and points nobody depends on are F
 __global__ void k_pmis_init(int n, const int* rp, const uint8_t* S, const int* cnt, unsigned long long seed,
-                            int level, double* w, signed char* CF) {
+                            int level, JointOff rows, double* w, signed char* CF) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  double u = splitmix_uniform(seed, 1000ULL + (uint64_t)level, (uint64_t)i);
+  double u = splitmix_uniform(seed, 1000ULL + (uint64_t)level, (uint64_t)(i - rows.off[joint_of(rows, i)]));
   double wi = __dadd_rn((double)cnt[i], u);
   w[i] = wi;
   int ns = 0;
@@ -388,8 +404,8 @@ __global__ void k_pmis_init(int n, const int* rp, const uint8_t* S, const int* c
 }
 
 void launch_pmis_init(int n, const int* rp, const uint8_t* S, const int* cnt, unsigned long long seed, int level,
-                      double* w, signed char* CF, cudaStream_t s) {
-  k_pmis_init<<<cdiv(n, kThreads), kThreads, 0, s>>>(n, rp, S, cnt, seed, level, w, CF);
+                      const JointOff& rows, double* w, signed char* CF, cudaStream_t s) {
+  k_pmis_init<<<cdiv(n, kThreads), kThreads, 0, s>>>(n, rp, S, cnt, seed, level, rows, w, CF);
   MGD_LAUNCH_CHECK();
 }
 
@@ -1571,27 +1587,32 @@ __global__ void k_dense_inverse(int n, double* a, int* piv, double* inv, double*
   }
 }
 
-// Gauss-Jordan on [A | I] in shared memory, one 1024-thread block (n <= kGjMax).
-// The rows below the pivot are updated exactly as the LU elimination above
-// does (l = a_ik / a_kk, a_ij -= l a_kj, no fused multiply-add in this unit),
-// so the pivot rows and the singularity decision are those of k_dense_inverse;
-// rows above the pivot are eliminated too, and the reduced rows are finally
-// divided by their pivots.
+// Gauss-Jordan on [A | I] in shared memory, one matrix per blockIdx.y, given in
+// CSR with local columns (n <= kGjMax).  The rows below the pivot are updated
+// exactly as the LU elimination above does (l = a_ik / a_kk, a_ij -= l a_kj, no
+// fused multiply-add in this unit), so the pivot rows and the singularity
+// decision are those of k_dense_inverse; rows above the pivot are eliminated
+// too, and the reduced rows are finally divided by their pivots.  The columns
+// of I are independent given the multipliers: kGjSlices blocks eliminate A
+// alike and each takes a share of them, because one SM's FP64 pipe is what the
+// elimination waits for (100 rows: 0.71 ms on one block).
 constexpr int kGjThreads = 1024;
-constexpr int kGjMax = 112;  // 2 n^2 doubles + n multipliers fit the opt-in shared memory
-__global__ void __launch_bounds__(kGjThreads) k_dense_inverse_gj(int n, const double* __restrict__ a0, int* piv,
-                                                                 double* inv, double* invT, int* status) {
+constexpr int kGjSlices = 6;
+__global__ void __launch_bounds__(kGjThreads) k_dense_inverse_gj(const InvDesc* __restrict__ descs, int* status) {
   extern __shared__ double gj[];
-  double* A = gj;          // n x n, row-major
-  double* X = gj + n * n;  // n x n, row-major, starts as I
-  double* L = X + n * n;   // multipliers of the current step
   __shared__ int s_pr;
   __shared__ double s_best;
-  const int t = threadIdx.x;
-  for (int e = t; e < n * n; e += kGjThreads) {
-    A[e] = a0[e];
-    X[e] = (e / n == e % n) ? 1.0 : 0.0;
-  }
+  const InvDesc d = descs[blockIdx.y];
+  const int n = d.n, t = threadIdx.x;
+  const int c0 = n * blockIdx.x / kGjSlices, nx = n * (blockIdx.x + 1) / kGjSlices - c0;  // columns of I
+  double* A = gj;           // n x n, row-major
+  double* X = gj + n * n;   // n x nx, row-major, starts as columns c0 .. of I
+  double* L = X + n * nx;   // multipliers of the current step
+  for (int e = t; e < n * n; e += kGjThreads) A[e] = 0.0;
+  for (int e = t; e < n * nx; e += kGjThreads) X[e] = (e / nx == c0 + e % nx) ? 1.0 : 0.0;
+  __syncthreads();
+  for (int i = t >> 5; i < n; i += kGjThreads / 32)
+    for (int p = d.rp[i] + (t & 31); p < d.rp[i + 1]; p += 32) A[i * n + d.ci[p]] = d.v[p];
   __syncthreads();
   for (int k = 0; k < n; ++k) {
     if (t < 32) {  // pivot: largest |a_ik|, i >= k, first index on ties (as the sequential search)
@@ -1616,7 +1637,6 @@ __global__ void __launch_bounds__(kGjThreads) k_dense_inverse_gj(int n, const do
       if (t == 0) {
         s_pr = pr;
         s_best = best;
-        piv[k] = pr;
       }
     }
     __syncthreads();
@@ -1625,20 +1645,20 @@ __global__ void __launch_bounds__(kGjThreads) k_dense_inverse_gj(int n, const do
       return;
     }
     const int pr = s_pr;
-    if (pr != k)
-      for (int j = t; j < 2 * n; j += kGjThreads) {
-        double* M = j < n ? A : X;
-        int c = j < n ? j : j - n;
-        double tmp = M[k * n + c];
-        M[k * n + c] = M[pr * n + c];
-        M[pr * n + c] = tmp;
+    if (pr != k && pr < n)
+      for (int j = t; j < n + nx; j += kGjThreads) {
+        double* M = j < n ? A + j : X + (j - n);
+        const int ld = j < n ? n : nx;
+        double tmp = M[k * ld];
+        M[k * ld] = M[pr * ld];
+        M[pr * ld] = tmp;
       }
     __syncthreads();
     for (int i = t; i < n; i += kGjThreads) L[i] = i == k ? 0.0 : __ddiv_rn(A[i * n + k], A[k * n + k]);
     __syncthreads();
     // every row but k: columns k+1.. of A and all of X (32 x 32 threads: rows by
     // thread row, columns by lane)
-    const int wa = n - k - 1, w = wa + n;
+    const int wa = n - k - 1, w = wa + nx;
     const int ty = t >> 5, tx = t & 31;
     for (int i = ty; i < n; i += kGjThreads / 32) {
       if (i == k) continue;
@@ -1649,31 +1669,32 @@ __global__ void __launch_bounds__(kGjThreads) k_dense_inverse_gj(int n, const do
           A[i * n + c] = __dsub_rn(A[i * n + c], __dmul_rn(li, A[k * n + c]));
         } else {
           int c = j - wa;
-          X[i * n + c] = __dsub_rn(X[i * n + c], __dmul_rn(li, X[k * n + c]));
+          X[i * nx + c] = __dsub_rn(X[i * nx + c], __dmul_rn(li, X[k * nx + c]));
         }
       }
     }
     __syncthreads();
   }
-  for (int e = t; e < n * n; e += kGjThreads) {
-    int i = e / n, c = e % n;
-    double v = __ddiv_rn(X[e], A[i * n + i]);
-    inv[e] = v;
-    invT[c * n + i] = v;
+  for (int e = t; e < n * nx; e += kGjThreads) {
+    const int i = e / nx, c = e % nx;
+    const double v = __ddiv_rn(X[e], A[i * n + i]);
+    d.inv[i * n + c0 + c] = v;
+    d.invT[(c0 + c) * n + i] = v;
   }
 }
 
+void launch_dense_inverses(const InvDesc* d, int nd, int maxn, int* status, cudaStream_t s) {
+  if (nd <= 0) return;
+  auto bytes = [](int n) { return (size_t)(n * n + n * cdiv(n, kGjSlices) + n) * sizeof(double); };
+  static const cudaError_t attr =
+      cudaFuncSetAttribute(k_dense_inverse_gj, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes(kGjMax));
+  MGD_CUDA(attr);
+  k_dense_inverse_gj<<<dim3(kGjSlices, nd), kGjThreads, bytes(maxn), s>>>(d, status);
+  MGD_LAUNCH_CHECK();
+}
+
+// one larger matrix (densified)
 void launch_dense_inverse(int n, double* a, int* piv, double* inv, double* invT, int* status, cudaStream_t s) {
-  if (n <= kGjMax) {
-    size_t smem = (size_t)(2 * n * n + n) * sizeof(double);
-    static const cudaError_t attr = cudaFuncSetAttribute(
-        k_dense_inverse_gj, cudaFuncAttributeMaxDynamicSharedMemorySize,
-        (int)((size_t)(2 * kGjMax * kGjMax + kGjMax) * sizeof(double)));
-    MGD_CUDA(attr);
-    k_dense_inverse_gj<<<1, kGjThreads, smem, s>>>(n, a, piv, inv, invT, status);
-    MGD_LAUNCH_CHECK();
-    return;
-  }
   k_dense_inverse<<<1, 128, 0, s>>>(n, a, piv, inv, invT, status);
   MGD_LAUNCH_CHECK();
 }
@@ -1763,18 +1784,20 @@ void launch_pctl_ac_fill(int N, int nc, int G, const int* const* brp, const int*
 }
 
 // ------------------------------------------------------------------ SELL-32 construction
-__global__ void k_sell_widths(int n, const int* rp, int* w) {
+__global__ void k_sell_widths(JointOff rows, JointOff slices, const int* rp, int* w) {
   int s = blockIdx.x * blockDim.x + threadIdx.x;
-  int nsl = (n + 31) / 32;
-  if (s >= nsl) return;
+  if (s >= slices.off[slices.n]) return;
+  const int k = joint_of(slices, s);
+  const int r0 = rows.off[k] + 32 * (s - slices.off[k]), r1 = min(rows.off[k + 1], r0 + 32);
   int mx = 0;
-  for (int r = s * 32; r < min(n, s * 32 + 32); ++r) mx = max(mx, rp[r + 1] - rp[r]);
+  for (int r = r0; r < r1; ++r) mx = max(mx, rp[r + 1] - rp[r]);
   w[s] = mx * 32;
 }
 
-void launch_sell_widths(int n, const int* rp, int* w, cudaStream_t s) {
-  int nsl = (n + 31) / 32;
-  k_sell_widths<<<cdiv(nsl, kThreads), kThreads, 0, s>>>(n, rp, w);
+void launch_sell_widths(const JointOff& rows, const JointOff& slices, const int* rp, int* w, cudaStream_t s) {
+  const int nsl = slices.off[slices.n];
+  if (nsl <= 0) return;
+  k_sell_widths<<<cdiv(nsl, kThreads), kThreads, 0, s>>>(rows, slices, rp, w);
   MGD_LAUNCH_CHECK();
 }
 
@@ -1782,23 +1805,27 @@ void launch_sell_widths(int n, const int* rp, int* w, cudaStream_t s) {
 // original index of a row of a row-permuted copy).  With d given, svpre gets
 // the column-scaled values a_ij d_j (A D^-1, rounded once in FP64, then to T).
 template <typename T>
-__global__ void k_sell_fill(int n, const int* rp, const int* ci, const double* v, const double* d,
-                            const int* sptr, int* sci, T* sv, T* svpre, const int* selfmap) {
-  int r = blockIdx.x * blockDim.x + threadIdx.x;
-  int nsl = (n + 31) / 32;
-  if (r >= nsl * 32) return;
-  int s = r >> 5, lane = r & 31;
-  int base = sptr[s];
-  int width = (sptr[s + 1] - base) >> 5;
-  int len = r < n ? rp[r + 1] - rp[r] : 0;
-  int b = r < n ? rp[r] : 0;
-  int self = r < n ? (selfmap ? selfmap[r] : r) : 0;
+__global__ void k_sell_fill(JointOff rows, JointOff slices, const int* rp, const int* ci, const double* v,
+                            const double* d, const int* sptr, int* sci, T* sv, T* svpre, unsigned vmask,
+                            const int* selfmap) {
+  const int g = blockIdx.x * blockDim.x + threadIdx.x;
+  const int s = g >> 5, lane = g & 31;
+  if (s >= slices.off[slices.n]) return;
+  const int k = joint_of(slices, s), row0 = rows.off[k];
+  const int r = row0 + 32 * (s - slices.off[k]) + lane;
+  const bool ok = r < rows.off[k + 1];
+  if (!(vmask >> k & 1u)) sv = nullptr;
+  const int base = sptr[s];
+  const int width = (sptr[s + 1] - base) >> 5;
+  const int b = ok ? rp[r] : 0;
+  const int len = ok ? rp[r + 1] - b : 0;
+  const int self = ok ? (selfmap ? selfmap[r] : r - row0) : 0;
   for (int j = 0; j < width; ++j) {
     int idx = base + j * 32 + lane;
     if (j < len) {
       int c = ci[b + j];
       double a = v[b + j];
-      sci[idx] = c;
+      sci[idx] = c - row0;
       if (sv) sv[idx] = (T)a;
       if (svpre) svpre[idx] = (T)__dmul_rn(a, d[c]);
     } else {
@@ -1810,32 +1837,94 @@ __global__ void k_sell_fill(int n, const int* rp, const int* ci, const double* v
 }
 
 template <typename T>
-static void sell_fill(int n, const int* rp, const int* ci, const double* v, const double* d, const int* sptr,
-                      int* sci, T* sv, T* svpre, cudaStream_t s, const int* selfmap) {
-  int nsl = (n + 31) / 32;
-  k_sell_fill<T><<<cdiv(nsl * 32, kThreads), kThreads, 0, s>>>(n, rp, ci, v, d, sptr, sci, sv, d ? svpre : nullptr,
-                                                               selfmap);
+void launch_sell_fill(const JointOff& rows, const JointOff& slices, const int* rp, const int* ci, const double* v,
+                      const double* d, const int* sptr, int* sci, T* sv, T* svpre, unsigned vmask, cudaStream_t s,
+                      const int* selfmap) {
+  const int nsl = slices.off[slices.n];
+  if (nsl <= 0) return;
+  k_sell_fill<T><<<cdiv(nsl * 32LL, kThreads), kThreads, 0, s>>>(rows, slices, rp, ci, v, d, sptr, sci, sv,
+                                                                 d ? svpre : nullptr, vmask, selfmap);
+  MGD_LAUNCH_CHECK();
+}
+template void launch_sell_fill<double>(const JointOff&, const JointOff&, const int*, const int*, const double*,
+                                       const double*, const int*, int*, double*, double*, unsigned, cudaStream_t,
+                                       const int*);
+template void launch_sell_fill<float>(const JointOff&, const JointOff&, const int*, const int*, const double*,
+                                      const double*, const int*, int*, float*, float*, unsigned, cudaStream_t,
+                                      const int*);
+
+// ------------------------------------------------------------------ joint matrices
+constexpr int kLocLanes = 8;  // lanes per row
+__global__ void k_localise(JointOff rows, JointOff cols, const int* rp, int* ci) {
+  const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const int r = (int)(g / kLocLanes), lane = (int)(g % kLocLanes);
+  if (r >= rows.off[rows.n]) return;
+  const int o = cols.off[joint_of(rows, r)];
+  if (o == 0) return;
+  for (int p = rp[r] + lane; p < rp[r + 1]; p += kLocLanes) ci[p] -= o;
+}
+
+void launch_localise(const JointOff& rows, const JointOff& cols, const int* rp, int* ci, cudaStream_t s) {
+  const int n = rows.off[rows.n];
+  if (n <= 0 || rows.n <= 1) return;
+  k_localise<<<cdiv((long long)n * kLocLanes, kThreads), kThreads, 0, s>>>(rows, cols, rp, ci);
   MGD_LAUNCH_CHECK();
 }
 
-void launch_sell_fill(int n, const int* rp, const int* ci, const double* v, const double* d, const int* sptr,
-                      int* sci, double* sv, double* svpre, cudaStream_t s, const int* selfmap) {
-  sell_fill<double>(n, rp, ci, v, d, sptr, sci, sv, svpre, s, selfmap);
+__global__ void k_join(int n, const int* rp, const int* ci, const double* v, int row0, int entry0, int* jrp, int* jci,
+                       double* jv) {
+  const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const int r = (int)(g / kLocLanes), lane = (int)(g % kLocLanes);
+  if (r >= n) return;
+  const int b = rp[r], e = rp[r + 1];
+  if (lane == 0) {
+    jrp[row0 + r] = entry0 + b;
+    if (r == n - 1) jrp[row0 + n] = entry0 + e;
+  }
+  for (int p = b + lane; p < e; p += kLocLanes) {
+    jci[entry0 + p] = ci[p] + row0;
+    jv[entry0 + p] = v[p];
+  }
 }
 
-void launch_sell_fill(int n, const int* rp, const int* ci, const double* v, const double* d, const int* sptr,
-                      int* sci, float* sv, float* svpre, cudaStream_t s, const int* selfmap) {
-  sell_fill<float>(n, rp, ci, v, d, sptr, sci, sv, svpre, s, selfmap);
+void launch_join(int n, const int* rp, const int* ci, const double* v, int row0, int entry0, int* jrp, int* jci,
+                 double* jv, cudaStream_t s) {
+  if (n <= 0) return;
+  k_join<<<cdiv((long long)n * kLocLanes, kThreads), kThreads, 0, s>>>(n, rp, ci, v, row0, entry0, jrp, jci, jv);
+  MGD_LAUNCH_CHECK();
+}
+
+__global__ void k_pick_ints(JointOff at, const int* src, int* out) {
+  if ((int)threadIdx.x <= at.n) out[threadIdx.x] = src[at.off[threadIdx.x]];
+}
+
+void launch_pick_ints(const JointOff& at, const int* src, int* out, cudaStream_t s) {
+  k_pick_ints<<<1, kMaxJoint + 32, 0, s>>>(at, src, out);
+  MGD_LAUNCH_CHECK();
+}
+
+__global__ void k_gather_ints(const int* const* src, int m, int* out) {
+  int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < m) out[i] = *src[i];
+}
+
+void launch_gather_ints(const int* const* src, int m, int* out, cudaStream_t s) {
+  if (m <= 0) return;
+  k_gather_ints<<<cdiv(m, kThreads), kThreads, 0, s>>>(src, m, out);
+  MGD_LAUNCH_CHECK();
 }
 
 // ------------------------------------------------------------------ Q = P - D^-1 A P
-// One block per 256-row window: each row's place in the window's order by
-// length (longest first, equal lengths by index; rows past n last), and the
-// width of each of its eight 32-row slices, the length of its first row.
-__global__ void __launch_bounds__(kQWin) k_q_order(int n, const int* rp, unsigned char* perm, int* widths) {
+// One block per 256-row window (windows do not cross operators): each row's
+// place in the window's order by length (longest first, equal lengths by
+// index; rows past the operator's last), and the width of each of its eight
+// 32-row slices, the length of its first row.
+__global__ void __launch_bounds__(kQWin) k_q_order(JointOff rows, JointOff wins, const int* rp, unsigned char* perm,
+                                                   int* widths) {
   __shared__ int s_len[kQWin];
-  const int t = threadIdx.x, r = blockIdx.x * kQWin + t;
-  const int len = r < n ? rp[r + 1] - rp[r] : -1;
+  const int k = joint_of(wins, blockIdx.x);
+  const int t = threadIdx.x, r = rows.off[k] + ((int)blockIdx.x - wins.off[k]) * kQWin + t;
+  const int len = r < rows.off[k + 1] ? rp[r + 1] - rp[r] : -1;
   s_len[t] = len;
   __syncthreads();
   int place = 0;
@@ -1847,42 +1936,47 @@ __global__ void __launch_bounds__(kQWin) k_q_order(int n, const int* rp, unsigne
   if ((place & 31) == 0) widths[blockIdx.x * (kQWin / 32) + (place >> 5)] = 32 * max(len, 0);
 }
 
-void launch_q_order(int n, const int* rp, unsigned char* perm, int* widths, cudaStream_t s) {
-  k_q_order<<<cdiv(n, kQWin), kQWin, 0, s>>>(n, rp, perm, widths);
+void launch_q_order(const JointOff& rows, const JointOff& wins, const int* rp, unsigned char* perm, int* widths,
+                    cudaStream_t s) {
+  if (wins.off[wins.n] <= 0) return;
+  k_q_order<<<wins.off[wins.n], kQWin, 0, s>>>(rows, wins, rp, perm, widths);
   MGD_LAUNCH_CHECK();
 }
 
 // The values of Q on the pattern of A P (its row i holds P's row i: a_ii is
 // stored): q_ic = p_ic - d_i (A P)_ic, in place in the CSR values and copied
-// to the sorted SELL-32 layout.  A thread per sorted place merges its rows of
-// A P and P, both in increasing column order.  Padding is a zero at the row's
-// first column.
+// to the sorted SELL-32 layout; columns become local to each operator (cols).
+// A thread per sorted place merges its rows of A P and P, both in increasing
+// column order.  Padding is a zero at the row's first column.
 template <typename T>
-__global__ void __launch_bounds__(kQWin) k_q_fill(int n, const int* rp, const int* ci, double* q, float* q32,
-                                                  const int* prp, const int* pci, const double* pv,
-                                                  const double* dinv, const unsigned char* perm, const int* sptr,
-                                                  int* sci, T* sv) {
+__global__ void __launch_bounds__(kQWin) k_q_fill(JointOff rows, JointOff cols, JointOff wins, const int* rp, int* ci,
+                                                  double* q, float* q32, const int* prp, const int* pci,
+                                                  const double* pv, const double* dinv, const unsigned char* perm,
+                                                  const int* sptr, int* sci, T* sv) {
+  const int k = joint_of(wins, blockIdx.x), c0 = cols.off[k];
   const int place = blockIdx.x * kQWin + threadIdx.x;
-  const int r = blockIdx.x * kQWin + perm[place];
+  const int r = rows.off[k] + ((int)blockIdx.x - wins.off[k]) * kQWin + perm[place];
   const int base = sptr[place >> 5], width = (sptr[(place >> 5) + 1] - base) >> 5;
   int b = 0, e = 0, pp = 0, pe = 0;
   double d = 0.0;
-  if (r < n) {
+  if (r < rows.off[k + 1]) {
     b = rp[r];
     e = rp[r + 1];
     pp = prp[r];
     pe = prp[r + 1];
     d = dinv[r];
   }
-  const int first = e > b ? ci[b] : 0;
+  const int first = e > b ? ci[b] - c0 : 0;
   for (int j = 0; j < width; ++j) {
     const size_t idx = (size_t)base + 32 * (size_t)j + (place & 31);
     int c = first;
     T out = T(0);
     if (b + j < e) {
-      c = ci[b + j];
+      const int jc = ci[b + j];
       double v = -__dmul_rn(d, q[b + j]);
-      if (pp < pe && pci[pp] == c) v = __dadd_rn(v, pv[pp++]);
+      if (pp < pe && pci[pp] == jc) v = __dadd_rn(v, pv[pp++]);
+      c = jc - c0;
+      ci[b + j] = c;
       q[b + j] = v;
       if (q32) q32[b + j] = (float)v;
       out = (T)v;
@@ -1893,18 +1987,20 @@ __global__ void __launch_bounds__(kQWin) k_q_fill(int n, const int* rp, const in
 }
 
 template <typename T>
-void launch_q_fill(int n, const int* rp, const int* ci, double* q, float* q32, const int* prp, const int* pci,
-                   const double* pv, const double* dinv, const unsigned char* perm, const int* sptr, int* sci, T* sv,
-                   cudaStream_t s) {
-  k_q_fill<T><<<cdiv(n, kQWin), kQWin, 0, s>>>(n, rp, ci, q, q32, prp, pci, pv, dinv, perm, sptr, sci, sv);
+void launch_q_fill(const JointOff& rows, const JointOff& cols, const JointOff& wins, const int* rp, int* ci, double* q,
+                   float* q32, const int* prp, const int* pci, const double* pv, const double* dinv,
+                   const unsigned char* perm, const int* sptr, int* sci, T* sv, cudaStream_t s) {
+  if (wins.off[wins.n] <= 0) return;
+  k_q_fill<T><<<wins.off[wins.n], kQWin, 0, s>>>(rows, cols, wins, rp, ci, q, q32, prp, pci, pv, dinv, perm, sptr, sci,
+                                                 sv);
   MGD_LAUNCH_CHECK();
 }
-template void launch_q_fill<double>(int, const int*, const int*, double*, float*, const int*, const int*,
-                                    const double*, const double*, const unsigned char*, const int*, int*, double*,
-                                    cudaStream_t);
-template void launch_q_fill<float>(int, const int*, const int*, double*, float*, const int*, const int*,
-                                   const double*, const double*, const unsigned char*, const int*, int*, float*,
-                                   cudaStream_t);
+template void launch_q_fill<double>(const JointOff&, const JointOff&, const JointOff&, const int*, int*, double*,
+                                    float*, const int*, const int*, const double*, const double*,
+                                    const unsigned char*, const int*, int*, double*, cudaStream_t);
+template void launch_q_fill<float>(const JointOff&, const JointOff&, const JointOff&, const int*, int*, double*,
+                                   float*, const int*, const int*, const double*, const double*,
+                                   const unsigned char*, const int*, int*, float*, cudaStream_t);
 
 // ------------------------------------------------------------------ column scaling A D^-1
 // out = A D^-1 values (the FP64 product, rounded to T); vout, when given, the

@@ -179,3 +179,30 @@ def test_dense_coarse_levels_match_oracle(gpu, orc, tmp_path):
                 lam = np.array(r["lam"])
                 assert np.linalg.norm(lam - lo) <= 1e-10 * np.linalg.norm(lo), (level, case)
     assert seen == {True, False}
+
+
+@pytest.mark.parametrize("kind,interp,prec", [("bd", 0, 0), ("schur2", 1, 0), ("schur1", 0, 1)])
+def test_joint_setup_many_operators(gpu, orc, kind, interp, prec):
+    # the most operators one joint setup takes (30 groups, E and I), of which E stalls at once and the others end on
+    # different levels: every level as the oracle sets it up alone, and the apply (bounds as above)
+    import torch
+    s = inputs.make_system(30, (23, 17), multigroup=True)
+    slv = gpu.Solver(batched=1, precision=prec, interp_type=interp, max_coarse=20).setup_system(s, kind)
+    M = orc.Block(orc.csr_of_system(s), s.G, s.N, kind, orc.opts(interp_type=interp, max_coarse=20))
+    depths = set()
+    for k in range(slv.stats()["n_ops"]):
+        info = slv.op_info(k)
+        h = M.amg(info["kind"], info["comp"])
+        assert info["nlevels"] == h.nlevels
+        depths.add(h.nlevels)
+        for l in range(h.nlevels):
+            g = slv.level(k, l)
+            for name, m in (("", h.A(l)), ("p", h.P(l) if l < h.nlevels - 1 else None)):
+                if m is not None:
+                    rp, ci, v = m.arrays()
+                    assert np.array_equal(g[name + "rp"], rp) and np.array_equal(g[name + "ci"], ci)
+                    assert np.array_equal(g[name + "v"], v), (k, l, name)
+    assert len(depths) > 1
+    z = slv.precond_apply(torch.from_numpy(s.b)).cpu().numpy()
+    zo = M.apply(s.b)
+    assert np.linalg.norm(z - zo) <= (1e-12 if prec == 0 else 1e-4) * np.linalg.norm(zo)
