@@ -21,6 +21,13 @@ struct XPlain {
   __device__ __forceinline__ T operator()(int j) const { return __ldg(x + j); }
 };
 
+// for a vector that the kernel also writes
+template <typename T>
+struct XCoherent {
+  const T* x;
+  __device__ __forceinline__ T operator()(int j) const { return x[j]; }
+};
+
 // Row dot product sum_p a_ip x(ci_p).  Every lane of the calling warp must
 // reach this function (shuffles); lanes whose row is out of range pass
 // valid = false and get 0.

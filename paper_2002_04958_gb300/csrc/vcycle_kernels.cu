@@ -492,22 +492,31 @@ template void launch_phase<float>(int, int, int, const LDesc<float>*, int, int, 
 // on these levels.
 template <typename T>
 __global__ void k_gs_first(const LDesc<T>* __restrict__ descs) {
-  MGD_PDL_ENTRY();
+  MGD_PDL_TRIGGER();
   const LDesc<T>* d = descs + blockIdx.y;
-  MGD_SKIP_INACTIVE(d);
   int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < d->n) d->xt[i] = d->key[i] == 0 ? d->b[i] * d->gdinv[i] : T(0);
+  if (i >= d->n) return;
+  const int key = d->key[i];
+  const T gd = d->gdinv[i];
+  MGD_PDL_WAIT();
+  MGD_SKIP_INACTIVE(d);
+  d->xt[i] = key == 0 ? d->b[i] * gd : T(0);
 }
 
 // step t of the down (up == 0: sweep t) or up (up == 1: sweep nk-1-t)
 // smoothing.  FMT_SELL reads the level's sweep-ordered SELL copy (coalesced
 // rows; position q of the sweep is row perm[q]); the CSR formats read A's
 // rows through perm with TPR threads per row.
+// A level has some 30 sweeps each way and a sweep few rows below the finest
+// levels, so what a launch waits for one after the other is its time: the
+// sweep's extent, its rows and their entries are setup data and are loaded
+// before the dependency wait (20 groups 256^2, levels of 39,540 to 3,886 rows:
+// 243 + 213 + 181 us a cycle with the loads
+// after it, 134 + 110 + 94 us so; level 0 330 -> 235 us).
 template <typename T, int FMT>
 __global__ void __launch_bounds__(kVThreads) k_gs_sweep(const LDesc<T>* __restrict__ descs, int t, int up) {
-  MGD_PDL_ENTRY();
+  MGD_PDL_TRIGGER();
   const LDesc<T>* d = descs + blockIdx.y;
-  MGD_SKIP_INACTIVE(d);
   if (FMT == FMT_SELL && d->gsptr == nullptr) return;  // no sweep-ordered copy (never planned so)
   constexpr int TPR = FmtTraits<FMT>::tpr;
   const int nk = d->nk;
@@ -520,10 +529,21 @@ __global__ void __launch_bounds__(kVThreads) k_gs_sweep(const LDesc<T>* __restri
   bool valid = idx < cnt;
   int q = seg + idx;
   int row = valid ? d->perm[q] : 0;
-  XPlain<T> xf{d->xt};
-  T s = FMT == FMT_SELL ? row_dot<T, FMT>(q, lane, valid, nullptr, nullptr, nullptr, d->gsptr, d->gsci, d->gsv, xf)
-                        : row_dot<T, FMT>(row, lane, valid, d->rp, d->ci, d->v, nullptr, nullptr, nullptr, xf);
-  if (valid && lane == 0) d->xt[row] = d->xt[row] + (d->b[row] - s) * d->gdinv[row];
+  RowPre<T, kPre> R;
+  if (FMT == FMT_SELL) row_load<T, FMT, kPre>(R, q, lane, valid, nullptr, nullptr, nullptr, d->gsptr, d->gsci, d->gsv);
+  else row_load<T, FMT, kPre>(R, row, lane, valid, d->rp, d->ci, d->v, nullptr, nullptr, nullptr);
+  const T gd = valid && lane == 0 ? d->gdinv[row] : T(0);
+  MGD_PDL_WAIT();
+  MGD_SKIP_INACTIVE(d);
+  T* const xt = d->xt;
+  XCoherent<T> xf{xt};  // xt is written by this launch's other points
+  T bi = T(0), xi = T(0);
+  if (valid && lane == 0) {
+    bi = d->b[row];
+    xi = xt[row];
+  }
+  T s = row_finish<T, FMT, kPre>(R, valid, d->ci, d->v, d->gsci, d->gsv, xf);
+  if (valid && lane == 0) xt[row] = xi + (bi - s) * gd;
 }
 
 // r = b - A xt after the down sweeps (the level's A layout)
