@@ -1642,6 +1642,9 @@ struct mgd_ctx {
   // FGMRES storage
   double *V = nullptr, *Z = nullptr, *w = nullptr, *r = nullptr, *hbuf = nullptr, *partial = nullptr,
          *ybuf = nullptr, *xtmp = nullptr, *btmp = nullptr;
+  double* krylov = nullptr;  // V and Z
+  size_t krylov_n = 0;
+  mgd::ScratchRegion* region = nullptr;  // setup scratch of the context stream, kept like the Krylov vectors
   double* hpin = nullptr;  // pinned host
   int m = 30;
   std::vector<double> hist;
@@ -1792,11 +1795,11 @@ static void finalize_op(mgd_ctx* c, InvOp& op, cudaStream_t st) {
 // jointly, in groups whose level-0 entries stay well inside 32-bit indices
 static void build_joint_ops(mgd_ctx* c, size_t first, size_t last) {
   SetupCtx sc{&c->ar, c->s, &c->o, mixed(c), c->o.keep_transpose != 0, &c->phases};
-  struct Region {  // setup scratch of the context stream
-    ScratchRegion r;
-    explicit Region(mgd_ctx* c) : r(c->s, c->ar.pool) { tl_region = &r; }
+  if (!c->region) c->region = new ScratchRegion(c->s, c->ar.pool);
+  struct Region {
+    explicit Region(ScratchRegion* r) { tl_region = r; }
     ~Region() { tl_region = nullptr; }
-  } region(c);
+  } region(c->region);
   std::vector<Hier*> hs;
   std::vector<const Csr*> as;
   long long nnz = 0;
@@ -2763,6 +2766,19 @@ static void capture_graph(mgd_ctx* c) {
   c->graph_ok = true;
 }
 
+static void free_region(mgd_ctx* c) {
+  delete c->region;
+  c->region = nullptr;
+  cudaStreamSynchronize(c->s);
+  if (c->ar.pool) cudaMemPoolTrimTo(c->ar.pool, 0);
+}
+
+static void free_krylov(mgd_ctx* c) {
+  if (c->krylov) cudaFreeAsync(c->krylov, c->s);
+  c->krylov = nullptr;
+  c->krylov_n = 0;
+}
+
 static void free_setup(mgd_ctx* c) {
   if (c->s) cudaStreamSynchronize(c->s);
   if (c->graph) cudaGraphExecDestroy(c->graph);
@@ -3073,8 +3089,21 @@ static void do_setup(mgd_ctx* c, const int* rp, const int* ci, const double* v, 
   pt_prog.stop();
   PhaseTimer pt_kry(&c->phases, SP_KRYLOV);
   c->m = std::max(1, std::min(o.restart, 30));
-  c->V = c->ar.alloc<double>((size_t)(c->m + 1) * n + kGsMaxUnit);  // every vector is written before it is read
-  c->Z = c->ar.alloc<double>((size_t)c->m * n);
+  // V and Z stay from setup to setup of one size (giving 9 GB back and taking it again costs the pool 5 ms); every
+  // vector is written before it is read
+  const size_t kn = (size_t)(2 * c->m + 1) * n + kGsMaxUnit;
+  if (c->krylov_n != kn) {
+    free_krylov(c);
+    try {
+      c->krylov = (double*)pool_alloc(c->ar.pool, sizeof(double) * kn, s);
+    } catch (const Error&) {  // short of memory: without the kept setup scratch
+      free_region(c);
+      c->krylov = (double*)pool_alloc(c->ar.pool, sizeof(double) * kn, s);
+    }
+    c->krylov_n = kn;
+  }
+  c->V = c->krylov;
+  c->Z = c->krylov + (size_t)(c->m + 1) * n + kGsMaxUnit;
   c->w = c->ar.alloc<double>(n, true);
   c->r = c->ar.alloc<double>(n, true);
   c->xtmp = c->ar.alloc<double>(n, true);
@@ -3842,6 +3871,8 @@ long long mgd_kernel_launches(void) { return __atomic_load_n(&g_kernel_launches,
 void mgd_destroy(mgd_ctx* c) {
   if (!c) return;
   free_setup(c);
+  free_krylov(c);
+  free_region(c);
   if (c->s_body) cudaStreamDestroy(c->s_body);
   for (auto cs : c->s_copy)
     if (cs) cudaStreamDestroy(cs);
