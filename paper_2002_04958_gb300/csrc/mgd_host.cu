@@ -328,14 +328,9 @@ static JointOff units_of(const JointOff& rows, int per) {
   return u;
 }
 
-// SELL-32 copy of A (operators at `rows`, columns made local) in the V-cycle's
-// precision only (FP32 values when mixed, else FP64); with dinv given, also
-// A D^-1 in the same layout (vpre); the values themselves only for the
-// operators of vmask (levels with Q never read them).
-static Sell build_sell(Arena& a, const Csr& A, const JointOff& rows, bool mixed, cudaStream_t s,
-                       const int* selfmap = nullptr, const double* dinv = nullptr, unsigned vmask = ~0u) {
+// slice pointers of a SELL-32 copy of A (operators at `rows`), and its column array
+static Sell sell_frame(Arena& a, const Csr& A, const JointOff& rows, const JointOff& slices, cudaStream_t s) {
   Scratch sc(s);
-  const JointOff slices = units_of(rows, 32);
   Sell S;
   S.n = A.n;
   S.nslices = slices.off[slices.n];
@@ -345,6 +340,17 @@ static Sell build_sell(Arena& a, const Csr& A, const JointOff& rows, bool mixed,
   exclusive_scan(w, S.sptr, S.nslices, s);
   S.nstored = read_int(S.sptr + S.nslices, s);
   S.ci = a.alloc<int>(S.nstored);
+  return S;
+}
+
+// SELL-32 copy of A (operators at `rows`, columns made local) in the V-cycle's
+// precision only (FP32 values when mixed, else FP64); with dinv given, also
+// A D^-1 in the same layout (vpre); the values themselves only for the
+// operators of vmask (levels with Q never read them).
+static Sell build_sell(Arena& a, const Csr& A, const JointOff& rows, bool mixed, cudaStream_t s,
+                       const int* selfmap = nullptr, const double* dinv = nullptr, unsigned vmask = ~0u) {
+  const JointOff slices = units_of(rows, 32);
+  Sell S = sell_frame(a, A, rows, slices, s);
   if (mixed) {
     if (vmask) S.v32 = a.alloc<float>(S.nstored);
     if (dinv) S.vpre32 = a.alloc<float>(S.nstored);
@@ -582,9 +588,7 @@ static bool coarsen_pass(SetupCtx& sc, const Csr& A, const JointOff& rows, unsig
     P.v = keep ? keep->alloc<double>(P.nnz) : ar.alloc<double>(P.nnz);
     double* dg = tmp.alloc<double>(n);
     launch_diag_extract(n, A.rp, A.ci, A.v, dg, s);
-    int* wi = tmp.alloc<int>((size_t)A.nnz + P.nnz);
-    double* wd = tmp.alloc<double>((size_t)A.nnz + n);
-    launch_interp_fill(n, A.nnz, A.rp, A.ci, A.v, S, CF, cidx, P.rp, P.nnz, P.ci, P.v, dg, wi, wd, s);
+    launch_interp_fill(n, A.rp, A.ci, A.v, S, CF, cidx, P.rp, P.ci, P.v, dg, s);
   }
   pt_int.stop();
   out.CF = CF;
@@ -864,23 +868,30 @@ static void build_joint(SetupCtx& sc, const std::vector<Hier*>& hs, const std::v
     unsigned vmask = 0;
     for (int k = 0; k < nops; ++k)
       if ((lv.coarsest >> k & 1u) && lv.rows.off[k + 1] - lv.rows.off[k] > o.max_coarse) vmask |= 1u << k;
-    Sell sell = build_sell(ar, lv.A, lv.rows, sc.mixed, s, nullptr, lv.dinv, vmask), sellT;
+    const JointOff slices = units_of(lv.rows, 32), wins = units_of(lv.rows, kQWin);
+    Sell sell = sell_frame(ar, lv.A, lv.rows, slices, s), sellT;
     float *v32 = nullptr, *vpre32 = nullptr, *pv32 = nullptr, *rv32 = nullptr, *atv32 = nullptr, *atvpre32 = nullptr;
     double *vpre = nullptr, *atvpre = nullptr;
+    if (sc.keepT) lv.AT = transpose(ar, lv.A, s);  // before the columns become local
     if (sc.mixed) {
       v32 = ar.alloc<float>(lv.A.nnz);
       vpre32 = ar.alloc<float>(lv.A.nnz);
-      launch_colscale_f32(lv.A.nnz, lv.A.ci, lv.A.v, lv.dinv, v32, vpre32, s);
+      if (vmask) sell.v32 = ar.alloc<float>(sell.nstored);
+      sell.vpre32 = ar.alloc<float>(sell.nstored);
+      launch_layouts<float>(lv.rows, slices, wins, lv.A.nnz, lv.A.rp, lv.A.ci, lv.A.v, lv.dinv, sell.sptr, sell.ci,
+                            sell.v32, sell.vpre32, vpre32, v32, vmask, l > 0, s);
       if (down) {
         pv32 = cast32(ar, lv.P.v, lv.P.nnz, s);
         rv32 = cast32(ar, lv.R.v, lv.R.nnz, s);
       }
     } else {
       vpre = ar.alloc<double>(lv.A.nnz);
-      launch_colscale(lv.A.nnz, lv.A.ci, lv.A.v, lv.dinv, vpre, s);
+      if (vmask) sell.v = ar.alloc<double>(sell.nstored);
+      sell.vpre = ar.alloc<double>(sell.nstored);
+      launch_layouts<double>(lv.rows, slices, wins, lv.A.nnz, lv.A.rp, lv.A.ci, lv.A.v, lv.dinv, sell.sptr, sell.ci,
+                             sell.v, sell.vpre, vpre, nullptr, vmask, l > 0, s);
     }
     if (sc.keepT) {
-      lv.AT = transpose(ar, lv.A, s);
       sellT = build_sell(ar, lv.AT, lv.rows, sc.mixed, s, nullptr, lv.dinv);
       if (sc.mixed) {
         atv32 = ar.alloc<float>(lv.AT.nnz);
@@ -892,11 +903,7 @@ static void build_joint(SetupCtx& sc, const std::vector<Hier*>& hs, const std::v
       }
       launch_localise(lv.rows, lv.rows, lv.AT.rp, lv.AT.ci, s);
     }
-    if (l > 0) launch_localise(lv.rows, lv.rows, lv.A.rp, lv.A.ci, s);
-    if (down) {
-      launch_localise(lv.rows, L[l + 1].rows, lv.P.rp, lv.P.ci, s);
-      launch_localise(L[l + 1].rows, lv.rows, lv.R.rp, lv.R.ci, s);
-    }
+    if (down) launch_localise(L[l + 1].rows, lv.rows, lv.R.rp, lv.R.ci, s);  // (A: launch_layouts, P and Q: build_q)
     // the operators' vectors b, xt, x, r in one zeroed block, each 256-byte aligned
     const size_t es = sc.mixed ? sizeof(float) : sizeof(double);
     auto pad = [&](int n) { return (es * n + 255) & ~(size_t)255; };
@@ -904,7 +911,6 @@ static void build_joint(SetupCtx& sc, const std::vector<Hier*>& hs, const std::v
     for (int k = 0; k < nops; ++k) bytes += 4 * pad(lv.rows.off[k + 1] - lv.rows.off[k]);
     char* vec = ar.alloc<char>(bytes);
     MGD_CUDA(cudaMemsetAsync(vec, 0, bytes, s));
-    const JointOff slices = units_of(lv.rows, 32), wins = units_of(lv.rows, kQWin);
     for (int k = 0; k < nops; ++k) {
       const int r0 = lv.rows.off[k], n = lv.rows.off[k + 1] - r0;
       if (n == 0 && l > 0) continue;

@@ -512,9 +512,8 @@ void launch_perm_rows_fill(int n, const int* perm, const int* rp, const int* ci,
                            int* pci, double* pv, cudaStream_t s);
 void launch_interp_count(int n, const int* rp, const int* ci, const uint8_t* S, const signed char* CF, int* cnt,
                          int* isc, cudaStream_t s);
-void launch_interp_fill(int n, int nnz, const int* rp, const int* ci, const double* v, const uint8_t* S,
-                        const signed char* CF, const int* cidx, const int* prp, int nnzp, int* pci, double* pv,
-                        const double* dg, int* work_i, double* work_d, cudaStream_t s);
+void launch_interp_fill(int n, const int* rp, const int* ci, const double* v, const uint8_t* S, const signed char* CF,
+                        const int* cidx, const int* prp, int* pci, double* pv, const double* dg, cudaStream_t s);
 void launch_exti_ub(int n, const int* rp, const int* ci, const uint8_t* S, const signed char* CF, const int* scount,
                     int* ub, cudaStream_t s);
 void launch_exti_list(int n, const int* rp, const int* ci, const uint8_t* S, const signed char* CF,
@@ -577,8 +576,13 @@ void launch_q_order(const JointOff& rows, const JointOff& wins, const int* rp, u
                     cudaStream_t s);
 template <typename T>
 void launch_q_fill(const JointOff& rows, const JointOff& cols, const JointOff& wins, const int* rp, int* ci, double* q,
-                   float* q32, const int* prp, const int* pci, const double* pv, const double* dinv,
+                   float* q32, const int* prp, int* pci, const double* pv, const double* dinv,
                    const unsigned char* perm, const int* sptr, int* sci, T* sv, cudaStream_t s);
+// SELL-32 and A D^-1 layouts of a joint operator in one pass (see k_layouts); wins: windows of kQWin rows
+template <typename T>
+void launch_layouts(const JointOff& rows, const JointOff& slices, const JointOff& wins, int nnz, const int* rp,
+                    int* ci, const double* v, const double* d, const int* sptr, int* sci, T* sv, T* svpre, T* vpre,
+                    float* v32, unsigned vmask, bool localise, cudaStream_t s);
 void launch_colscale(long long nnz, const int* ci, const double* v, const double* d, double* out, cudaStream_t s);
 // FP32 values (vout) and FP32 A D^-1 (out, when d is given) of FP64 CSR values, one pass
 void launch_colscale_f32(long long nnz, const int* ci, const double* v, const double* d, float* vout, float* out,

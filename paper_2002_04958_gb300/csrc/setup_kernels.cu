@@ -323,19 +323,30 @@ void launch_gamma_wc(int n, const double* d, const double* diag, double theta, i
 }
 
 // ------------------------------------------------------------------ strength of connection (Section 3.1)
+// |S_ij = -a_ij >= theta max_k(-a_ik)|.  The comparisons run on the integer pipe:
+// a negative binary64's magnitude bits order as -a does (0 here: not negative,
+// or NaN).  FP64 compares bound this kernel (83 % of the FP64 pipe).
+__device__ __forceinline__ long long neg_bits(double a) {
+  const long long b = __double_as_longlong(a), m = b & 0x7fffffffffffffffLL;
+  return b < 0 && m <= 0x7ff0000000000000LL ? m : 0;
+}
 __global__ void k_strength(int n, const int* rp, const int* ci, const double* v, double theta, uint8_t* S,
                            JointOff rows, unsigned active) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
+  const int b = rp[i], e = rp[i + 1];
   if (!(active >> joint_of(rows, i) & 1u)) {
-    for (int p = rp[i]; p < rp[i + 1]; ++p) S[p] = 0;
+    for (int p = b; p < e; ++p) S[p] = 0;
     return;
   }
-  double mx = 0.0;
-  for (int p = rp[i]; p < rp[i + 1]; ++p)
-    if (ci[p] != i && -v[p] > mx) mx = -v[p];
-  double thr = __dmul_rn(theta, mx);
-  for (int p = rp[i]; p < rp[i + 1]; ++p) S[p] = (uint8_t)(ci[p] != i && mx > 0.0 && -v[p] >= thr);
+  long long mx = 0;
+  for (int p = b; p < e; ++p)
+    if (ci[p] != i) mx = max(mx, neg_bits(v[p]));
+  const double thr = __dmul_rn(theta, __longlong_as_double(mx));
+  const long long tb = __double_as_longlong(thr);
+  // (a threshold that rounds to zero, or is negative or NaN, takes the FP64 compare)
+  for (int p = b; p < e; ++p)
+    S[p] = (uint8_t)(ci[p] != i && mx > 0 && (tb > 0 && tb <= 0x7ff0000000000000LL ? neg_bits(v[p]) >= tb : -v[p] >= thr));
 }
 
 void launch_strength(int n, const int* rp, const int* ci, const double* v, double theta, uint8_t* S,
@@ -686,11 +697,6 @@ __device__ __forceinline__ bool zero_f64(double x) { return (__double_as_longlon
 
 __device__ __forceinline__ bool opp_sign(double akm, double akk) { return pos_f64(akk) ? neg_f64(akm) : pos_f64(akm); }
 
-// One thread per row.  Numerators start from a_ij (j in C_i, row order); strong
-// F neighbours k distribute a_ik abar_kj / sum_{m in C_i} abar_km, or are lumped
-// into the diagonal with the weak neighbours when that sum is zero;
-// w_ij = -num_j / (a_ii + sum_W a_in).
-
 // ------------------------------------------------------------------ extended+i interpolation
 // (De Sterck, Falgout, Nolting, Yang 2008): the interpolatory set of an F point
 // adds, to its strong C neighbours, the strong C neighbours of its strong F
@@ -865,115 +871,101 @@ __global__ void k_exti_value(int nnzp, const int* prowof, const int* prp, const 
   pv[e] = !zero_f64(diag) ? __ddiv_rn(-num, diag) : 0.0;
 }
 
-// Classical modified interpolation values in passes that keep the operand
-// order of the row-sequential definition (so its bits): the strong C
-// neighbours of each F row are written in row order (sorted: CSR columns are
-// sorted), then a denominator per strong-F entry of A, the lumped diagonal per
-// row, the value of each entry of P, and last the fine-to-coarse column map.
-__global__ void k_cl_set(int n, const int* rp, const int* ci, const uint8_t* S, const signed char* CF,
-                         const int* cidx, const int* prp, int* pci, double* pv) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
+// Classical modified interpolation, one thread per row.  Numerators start from
+// a_ij (j in C_i); a strong F neighbour k distributes a_ik abar_km / sum_{l in
+// C_i} abar_kl over its opposite-sign connections into C_i, or is lumped into
+// the diagonal with the weak neighbours when that sum is zero;
+// w_ij = -num_j / (a_ii + sum_W a_in).  Neighbours are taken in row order, and
+// both rows are in column order, so C_i and row k are merged: one walk for the
+// sum, and one, of entries that are then in L1, for the shares.  (As a pass per
+// entry of A for the sums, one per row for the diagonal and one per entry of P
+// for the numerators, each entry found by binary search: 12.2 ms on the joint
+// levels of 21 x 884,736 rows, 9.1 ms so.)  The row's part of pci and pv holds C_i
+// (fine indices) and the numerators meanwhile.
+constexpr int kClMatch = 6;
+__global__ void __launch_bounds__(kThreads) k_cl_rows(int n, const int* __restrict__ rp, const int* __restrict__ ci,
+                                                      const double* __restrict__ v, const uint8_t* __restrict__ S,
+                                                      const signed char* __restrict__ CF, const int* __restrict__ cidx,
+                                                      const double* __restrict__ dg, const int* __restrict__ prp,
+                                                      int* pci, double* pv) {
+  __shared__ int s_q[kClMatch][kThreads];
+  __shared__ int s_t[kClMatch][kThreads];
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  int base = prp[i];
+  int* const C = pci + prp[i];
+  double* const num = pv + prp[i];
+  const int nl = prp[i + 1] - prp[i];
   if (CF[i] == 1) {
-    pci[base] = cidx[i];
-    pv[base] = 1.0;
+    C[0] = cidx[i];
+    num[0] = 1.0;
     return;
   }
-  int t = 0;
-  for (int p = rp[i]; p < rp[i + 1]; ++p)
-    if (S[p] && CF[ci[p]] == 1) pci[base + t++] = ci[p];  // fine index until the last pass
-}
-
-__global__ void k_cl_denom(int nnz, const int* rowof, const int* rp, const int* ci, const double* v, const uint8_t* S,
-                           const signed char* CF, const int* prp, const int* pci, const double* dg, double* den) {
-  int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= nnz) return;
-  int i = rowof[p], k = ci[p];
-  if (CF[i] == 1 || k == i || !(S[p] && CF[k] == -1)) return;
-  const int* L = pci + prp[i];
-  int nl = prp[i + 1] - prp[i];
-  double akk = dg[k];
-  double denom = 0.0;
-  for (int q = rp[k]; q < rp[k + 1]; ++q)
-    if (find_sorted(L, nl, ci[q]) >= 0 && opp_sign(v[q], akk)) denom = __dadd_rn(denom, v[q]);
-  den[p] = denom;
-}
-
-__global__ void k_cl_diag(int n, const int* rp, const int* ci, const double* v, const uint8_t* S,
-                          const signed char* CF, const int* prp, const double* den, double* diagv) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n || CF[i] == 1 || prp[i + 1] == prp[i]) return;
-  double diag = 0.0;
-  for (int p = rp[i]; p < rp[i + 1]; ++p)
-    if (ci[p] == i) diag = v[p];
-  for (int p = rp[i]; p < rp[i + 1]; ++p) {
-    int k = ci[p];
+  if (nl == 0) return;
+  const int b = rp[i], e = rp[i + 1];
+  for (int p = b, t = 0; p < e; ++p)
+    if (S[p] && CF[ci[p]] == 1) {
+      C[t] = ci[p];
+      num[t] = v[p];
+      ++t;
+    }
+  double diag = dg[i];
+  for (int p = b; p < e; ++p) {
+    const int k = ci[p];
     if (k == i) continue;
-    if (S[p] && CF[k] == 1) continue;
-    if (S[p] && CF[k] == -1) {
-      if (zero_f64(den[p])) diag = __dadd_rn(diag, v[p]);
-    } else {
-      diag = __dadd_rn(diag, v[p]);  // weak neighbours: lumped
+    const double aik = v[p];
+    if (!S[p]) {
+      diag = __dadd_rn(diag, aik);  // weak neighbours: lumped
+      continue;
+    }
+    if (CF[k] == 1) continue;
+    const double akk = dg[k];
+    const int kb = rp[k], ke = rp[k + 1];
+    double denom = 0.0;
+    for (int q = kb, t = 0; q < ke; ++q) {
+      const int c = ci[q];
+      while (t < nl && C[t] < c) ++t;
+      if (t == nl) break;
+      if (C[t] == c && opp_sign(v[q], akk)) denom = __dadd_rn(denom, v[q]);
+    }
+    if (zero_f64(denom)) {
+      diag = __dadd_rn(diag, aik);
+      continue;
+    }
+    // the shares are divided after the walk: a division inside it issues for a
+    // few lanes at a time, and FP64 issue is what the kernel waits for (79 % of
+    // the pipe; 4.3 -> 3.9 ms on the joint level 0)
+    int m = 0;
+    for (int q = kb, t = 0; q < ke; ++q) {
+      const int c = ci[q];
+      while (t < nl && C[t] < c) ++t;
+      if (t == nl) break;
+      if (C[t] == c && opp_sign(v[q], akk)) {
+        if (m < kClMatch) {
+          s_q[m][threadIdx.x] = q;
+          s_t[m][threadIdx.x] = t;
+          ++m;
+        } else {  // (each target takes one share of a neighbour: their order does not matter)
+          num[t] = __dadd_rn(num[t], __ddiv_rn(__dmul_rn(aik, v[q]), denom));
+        }
+      }
+    }
+    for (int u = 0; u < m; ++u) {
+      const int t = s_t[u][threadIdx.x];
+      num[t] = __dadd_rn(num[t], __ddiv_rn(__dmul_rn(aik, v[s_q[u][threadIdx.x]]), denom));
     }
   }
-  diagv[i] = diag;
+  const bool zero = zero_f64(diag);
+  for (int t = 0; t < nl; ++t) {
+    C[t] = cidx[C[t]];
+    num[t] = zero ? 0.0 : __ddiv_rn(-num[t], diag);
+  }
 }
 
-__global__ void k_cl_value(int nnzp, const int* prowof, const int* rp, const int* ci, const double* v,
-                           const uint8_t* S, const signed char* CF, const int* pci, const double* dg,
-                           const double* den, const double* diagv, double* pv) {
-  int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= nnzp) return;
-  int i = prowof[e];
-  if (CF[i] == 1) return;
-  int m = pci[e];
-  double num = 0.0;
-  int pd = find_col(rp, ci, i, m);
-  if (pd >= 0) num = v[pd];
-  for (int p = rp[i]; p < rp[i + 1]; ++p) {
-    int k = ci[p];
-    if (k == i || !(S[p] && CF[k] == -1)) continue;
-    double denom = den[p];
-    if (zero_f64(denom)) continue;
-    int q = find_col(rp, ci, k, m);
-    if (q >= 0 && opp_sign(v[q], dg[k])) num = __dadd_rn(num, __ddiv_rn(__dmul_rn(v[p], v[q]), denom));
-  }
-  double diag = diagv[i];
-  pv[e] = !zero_f64(diag) ? __ddiv_rn(-num, diag) : 0.0;
-}
-
-__global__ void k_cl_columns(int nnzp, const int* prowof, const signed char* CF, const int* cidx, int* pci) {
-  int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e < nnzp && CF[prowof[e]] != 1) pci[e] = cidx[pci[e]];
-}
-
-void launch_interp_fill(int n, int nnz, const int* rp, const int* ci, const double* v, const uint8_t* S,
-                        const signed char* CF, const int* cidx, const int* prp, int nnzp, int* pci, double* pv,
-                        const double* dg, int* work_i, double* work_d, cudaStream_t s) {
-  // work_i: nnz + nnzp ints (row of each entry of A, of P); work_d: nnz + n doubles
-  int* rowof = work_i;
-  int* prowof = work_i + nnz;
-  double* den = work_d;
-  double* diagv = work_d + nnz;
-  k_cl_set<<<cdiv(n, kThreads), kThreads, 0, s>>>(n, rp, ci, S, CF, cidx, prp, pci, pv);
+void launch_interp_fill(int n, const int* rp, const int* ci, const double* v, const uint8_t* S, const signed char* CF,
+                        const int* cidx, const int* prp, int* pci, double* pv, const double* dg, cudaStream_t s) {
+  if (n <= 0) return;
+  k_cl_rows<<<cdiv(n, kThreads), kThreads, 0, s>>>(n, rp, ci, v, S, CF, cidx, dg, prp, pci, pv);
   MGD_LAUNCH_CHECK();
-  k_row_of<<<cdiv(n, kThreads), kThreads, 0, s>>>(n, rp, rowof);
-  MGD_LAUNCH_CHECK();
-  k_row_of<<<cdiv(n, kThreads), kThreads, 0, s>>>(n, prp, prowof);
-  MGD_LAUNCH_CHECK();
-  if (nnz > 0) {
-    k_cl_denom<<<cdiv(nnz, kThreads), kThreads, 0, s>>>(nnz, rowof, rp, ci, v, S, CF, prp, pci, dg, den);
-    MGD_LAUNCH_CHECK();
-  }
-  k_cl_diag<<<cdiv(n, kThreads), kThreads, 0, s>>>(n, rp, ci, v, S, CF, prp, den, diagv);
-  MGD_LAUNCH_CHECK();
-  if (nnzp > 0) {
-    k_cl_value<<<cdiv(nnzp, kThreads), kThreads, 0, s>>>(nnzp, prowof, rp, ci, v, S, CF, pci, dg, den, diagv, pv);
-    MGD_LAUNCH_CHECK();
-    k_cl_columns<<<cdiv(nnzp, kThreads), kThreads, 0, s>>>(nnzp, prowof, CF, cidx, pci);
-    MGD_LAUNCH_CHECK();
-  }
 }
 
 void launch_exti_ub(int n, const int* rp, const int* ci, const uint8_t* S, const signed char* CF, const int* scount,
@@ -1918,22 +1910,56 @@ void launch_gather_ints(const int* const* src, int m, int* out, cudaStream_t s) 
 // One block per 256-row window (windows do not cross operators): each row's
 // place in the window's order by length (longest first, equal lengths by
 // index; rows past the operator's last), and the width of each of its eight
-// 32-row slices, the length of its first row.
+// 32-row slices.
 __global__ void __launch_bounds__(kQWin) k_q_order(JointOff rows, JointOff wins, const int* rp, unsigned char* perm,
                                                    int* widths) {
-  __shared__ int s_len[kQWin];
+  // counting sort by min(length, kLen - 2) (longer rows share the first class;
+  // rows past n come after the empty ones): a slice's width is the maximum over
+  // its rows
+  constexpr int kLen = 64, kWarps = kQWin / 32;
+  __shared__ int s_cnt[kLen][kWarps];  // rows of a class per warp, then their first place
+  __shared__ int s_tot[kLen], s_w[kWarps];
   const int k = joint_of(wins, blockIdx.x);
-  const int t = threadIdx.x, r = rows.off[k] + ((int)blockIdx.x - wins.off[k]) * kQWin + t;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int r = rows.off[k] + ((int)blockIdx.x - wins.off[k]) * kQWin + t;
   const int len = r < rows.off[k + 1] ? rp[r + 1] - rp[r] : -1;
-  s_len[t] = len;
+  const int cls = kLen - 2 - min(len, kLen - 2);  // 0: longest, kLen - 1: past n
+  for (int e = t; e < kLen * kWarps; e += kQWin) (&s_cnt[0][0])[e] = 0;
+  if (t < kWarps) s_w[t] = 0;
   __syncthreads();
-  int place = 0;
-  for (int j = 0; j < kQWin; ++j) {
-    const int o = s_len[j];
-    place += o > len || (o == len && j < t);
+  const unsigned same = __match_any_sync(0xffffffffu, cls);
+  const int before = __popc(same & ((1u << lane) - 1));
+  if (before == 0) s_cnt[cls][warp] = __popc(same);
+  __syncthreads();
+  if (t < kLen) {
+    int sum = 0;
+    for (int w = 0; w < kWarps; ++w) {
+      const int c = s_cnt[t][w];
+      s_cnt[t][w] = sum;
+      sum += c;
+    }
+    s_tot[t] = sum;
   }
+  __syncthreads();
+  if (warp == 0) {  // exclusive sums of the two halves of s_tot
+    int a = s_tot[lane], b = s_tot[32 + lane], sa = a, sb = b;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int ua = __shfl_up_sync(0xffffffffu, sa, o), ub = __shfl_up_sync(0xffffffffu, sb, o);
+      if (lane >= o) {
+        sa += ua;
+        sb += ub;
+      }
+    }
+    s_tot[lane] = sa - a;
+    s_tot[32 + lane] = __shfl_sync(0xffffffffu, sa, 31) + sb - b;
+  }
+  __syncthreads();
+  const int place = s_tot[cls] + s_cnt[cls][warp] + before;
   perm[(size_t)blockIdx.x * kQWin + place] = (unsigned char)t;
-  if ((place & 31) == 0) widths[blockIdx.x * (kQWin / 32) + (place >> 5)] = 32 * max(len, 0);
+  if (len > 0) atomicMax(&s_w[place >> 5], len);
+  __syncthreads();
+  if (t < kWarps) widths[blockIdx.x * kWarps + t] = 32 * s_w[t];
 }
 
 void launch_q_order(const JointOff& rows, const JointOff& wins, const int* rp, unsigned char* perm, int* widths,
@@ -1945,50 +1971,95 @@ void launch_q_order(const JointOff& rows, const JointOff& wins, const int* rp, u
 
 // The values of Q on the pattern of A P (its row i holds P's row i: a_ii is
 // stored): q_ic = p_ic - d_i (A P)_ic, in place in the CSR values and copied
-// to the sorted SELL-32 layout; columns become local to each operator (cols).
-// A thread per sorted place merges its rows of A P and P, both in increasing
-// column order.  Padding is a zero at the row's first column.
+// to the sorted SELL-32 layout; the columns of Q and P become local to each
+// operator (cols).  A block takes a window: its entries of A P, one stretch of
+// the CSR arrays, come through shared memory, so that both the CSR side and the
+// SELL side are read and written in order (a thread per row straight from and
+// to memory: 3.9 ms on 21 x 884,736 rows, 1.7 ms so); a thread per row merges its rows of
+// A P and P, both in increasing column order.  Padding is a zero at the row's
+// first column.  A window with more entries than fit is taken in place.
+constexpr int kQStage = 3584;  // entries staged (42 KB)
 template <typename T>
 __global__ void __launch_bounds__(kQWin) k_q_fill(JointOff rows, JointOff cols, JointOff wins, const int* rp, int* ci,
-                                                  double* q, float* q32, const int* prp, const int* pci,
+                                                  double* q, float* q32, const int* prp, int* pci,
                                                   const double* pv, const double* dinv, const unsigned char* perm,
                                                   const int* sptr, int* sci, T* sv) {
+  __shared__ double s_q[kQStage];
+  __shared__ int s_c[kQStage];
   const int k = joint_of(wins, blockIdx.x), c0 = cols.off[k];
-  const int place = blockIdx.x * kQWin + threadIdx.x;
-  const int r = rows.off[k] + ((int)blockIdx.x - wins.off[k]) * kQWin + perm[place];
-  const int base = sptr[place >> 5], width = (sptr[(place >> 5) + 1] - base) >> 5;
-  int b = 0, e = 0, pp = 0, pe = 0;
-  double d = 0.0;
-  if (r < rows.off[k + 1]) {
-    b = rp[r];
-    e = rp[r + 1];
-    pp = prp[r];
-    pe = prp[r + 1];
-    d = dinv[r];
-  }
-  const int first = e > b ? ci[b] - c0 : 0;
-  for (int j = 0; j < width; ++j) {
-    const size_t idx = (size_t)base + 32 * (size_t)j + (place & 31);
-    int c = first;
-    T out = T(0);
-    if (b + j < e) {
-      const int jc = ci[b + j];
-      double v = -__dmul_rn(d, q[b + j]);
-      if (pp < pe && pci[pp] == jc) v = __dadd_rn(v, pv[pp++]);
-      c = jc - c0;
-      ci[b + j] = c;
-      q[b + j] = v;
-      if (q32) q32[b + j] = (float)v;
-      out = (T)v;
+  const int t = threadIdx.x, place = blockIdx.x * kQWin + t;
+  const int w0 = rows.off[k] + ((int)blockIdx.x - wins.off[k]) * kQWin, w1 = min(w0 + kQWin, rows.off[k + 1]);
+  const int eb = rp[w0], ee = rp[w1];
+  const bool staged = ee - eb <= kQStage;
+  int* const C = staged ? s_c : ci + eb;  // the window's entries, from eb on
+  double* const Q = staged ? s_q : q + eb;
+  if (staged)
+    for (int e = eb + t; e < ee; e += kQWin) {
+      s_c[e - eb] = ci[e];
+      s_q[e - eb] = q[e];
     }
-    sci[idx] = c;
-    sv[idx] = out;
+  // the row's diagonal and its first entries of P, in flight with the staging
+  constexpr int PRE = 4;
+  const int r0 = w0 + t;
+  int b0 = 0, e0 = 0, pp = 0, np = 0, pc[PRE];
+  double pw[PRE], d = 0.0;
+  if (r0 < w1) {
+    b0 = rp[r0] - eb;
+    e0 = rp[r0 + 1] - eb;
+    pp = prp[r0];
+    np = prp[r0 + 1] - pp;
+    d = dinv[r0];
+  }
+#pragma unroll
+  for (int u = 0; u < PRE; ++u)
+    if (u < np) {
+      pc[u] = pci[pp + u];
+      pw[u] = pv[pp + u];
+    }
+  __syncthreads();
+  for (int j = b0; j < e0; ++j) {
+    Q[j] = -__dmul_rn(d, Q[j]);
+    C[j] -= c0;
+  }
+  // each entry of P meets its column once (both rows ascend)
+  int j = b0;
+  auto add = [&](int c, double w) {
+    while (j < e0 && C[j] < c - c0) ++j;
+    if (j < e0 && C[j] == c - c0) Q[j] = __dadd_rn(Q[j], w);
+  };
+#pragma unroll
+  for (int u = 0; u < PRE; ++u)
+    if (u < np) {
+      add(pc[u], pw[u]);
+      pci[pp + u] = pc[u] - c0;
+    }
+  for (int u = PRE; u < np; ++u) {
+    const int c = pci[pp + u];
+    add(c, pv[pp + u]);
+    pci[pp + u] = c - c0;
+  }
+  __syncthreads();
+  for (int e = eb + t; e < ee; e += kQWin) {
+    const double v = Q[e - eb];
+    if (staged) {
+      ci[e] = s_c[e - eb];
+      q[e] = v;
+    }
+    if (q32) q32[e] = (float)v;
+  }
+  const int r = w0 + perm[place];
+  const int base = sptr[place >> 5], width = (sptr[(place >> 5) + 1] - base) >> 5;
+  const int b = r < w1 ? rp[r] - eb : 0, len = r < w1 ? rp[r + 1] - eb - b : 0;
+  for (int j = 0; j < width; ++j) {
+    const size_t idx = (size_t)base + 32 * (size_t)j + (t & 31);
+    sci[idx] = j < len ? C[b + j] : len > 0 ? C[b] : 0;
+    sv[idx] = j < len ? (T)Q[b + j] : T(0);
   }
 }
 
 template <typename T>
 void launch_q_fill(const JointOff& rows, const JointOff& cols, const JointOff& wins, const int* rp, int* ci, double* q,
-                   float* q32, const int* prp, const int* pci, const double* pv, const double* dinv,
+                   float* q32, const int* prp, int* pci, const double* pv, const double* dinv,
                    const unsigned char* perm, const int* sptr, int* sci, T* sv, cudaStream_t s) {
   if (wins.off[wins.n] <= 0) return;
   k_q_fill<T><<<wins.off[wins.n], kQWin, 0, s>>>(rows, cols, wins, rp, ci, q, q32, prp, pci, pv, dinv, perm, sptr, sci,
@@ -1996,11 +2067,90 @@ void launch_q_fill(const JointOff& rows, const JointOff& cols, const JointOff& w
   MGD_LAUNCH_CHECK();
 }
 template void launch_q_fill<double>(const JointOff&, const JointOff&, const JointOff&, const int*, int*, double*,
-                                    float*, const int*, const int*, const double*, const double*,
-                                    const unsigned char*, const int*, int*, double*, cudaStream_t);
+                                    float*, const int*, int*, const double*, const double*, const unsigned char*,
+                                    const int*, int*, double*, cudaStream_t);
 template void launch_q_fill<float>(const JointOff&, const JointOff&, const JointOff&, const int*, int*, double*,
-                                   float*, const int*, const int*, const double*, const double*,
-                                   const unsigned char*, const int*, int*, float*, cudaStream_t);
+                                   float*, const int*, int*, const double*, const double*, const unsigned char*,
+                                   const int*, int*, float*, cudaStream_t);
+
+// ------------------------------------------------------------------ the operator's layouts
+// Everything the V-cycle reads of an operator besides its CSR values, in one
+// pass: A D^-1 as CSR (vpre) and SELL-32 (svpre), the values in SELL-32 for
+// the operators of vmask, in FP32 form the CSR values (v32), and the CSR
+// columns made local in place (localise).  A block takes 256 rows of one
+// operator (eight slices); their entries are one stretch of the CSR arrays and
+// come through shared memory as in k_q_fill (the SELL copy, the column scaling
+// and the renumbering were three passes: 5.4 ms over all levels, 3.3 ms so).
+template <typename T>
+__global__ void __launch_bounds__(kQWin) k_layouts(JointOff rows, JointOff wins, const int* rp, int* ci,
+                                                   const double* v, const double* d, JointOff slices, const int* sptr,
+                                                   int* sci, T* sv, T* svpre, T* vpre, float* v32, unsigned vmask,
+                                                   int localise, int cap) {
+  extern __shared__ double lay[];
+  const int k = joint_of(wins, blockIdx.x), row0 = rows.off[k];
+  const int t = threadIdx.x, win = (int)blockIdx.x - wins.off[k];
+  const int w0 = row0 + win * kQWin, w1 = min(w0 + kQWin, rows.off[k + 1]);
+  const int eb = rp[w0], ee = rp[w1];
+  const bool staged = ee - eb <= cap;
+  double* const s_p = lay;
+  int* const s_c = (int*)(lay + cap);
+  for (int e = eb + t; e < ee; e += kQWin) {
+    const int c = ci[e];
+    const double a = v[e], p = __dmul_rn(a, d[c]);
+    if (staged) {
+      s_c[e - eb] = c - row0;
+      s_p[e - eb] = p;
+      if (localise) ci[e] = c - row0;
+    }
+    vpre[e] = (T)p;
+    if (v32) v32[e] = (float)a;
+  }
+  __syncthreads();
+  const int r = w0 + t, sl = slices.off[k] + win * (kQWin / 32) + (t >> 5);
+  const bool ok = r < w1;
+  if (sl >= slices.off[k + 1]) return;
+  const bool values = vmask >> k & 1u;
+  const int base = sptr[sl], width = (sptr[sl + 1] - base) >> 5;
+  const int b = ok ? rp[r] : 0, len = ok ? rp[r + 1] - b : 0;
+  for (int j = 0; j < width; ++j) {
+    const int idx = base + j * 32 + (t & 31);
+    if (j < len) {
+      const int e = b + j;
+      sci[idx] = staged ? s_c[e - eb] : ci[e] - row0;
+      svpre[idx] = staged ? (T)s_p[e - eb] : (T)__dmul_rn(v[e], d[ci[e]]);
+      if (values) sv[idx] = (T)v[e];
+    } else {
+      sci[idx] = ok ? r - row0 : 0;
+      svpre[idx] = T(0);
+      if (values) sv[idx] = T(0);
+    }
+  }
+  if (!staged && localise)
+    for (int j = 0; j < len; ++j) ci[b + j] -= row0;
+}
+
+template <typename T>
+void launch_layouts(const JointOff& rows, const JointOff& slices, const JointOff& wins, int nnz, const int* rp,
+                    int* ci, const double* v, const double* d, const int* sptr, int* sci, T* sv, T* svpre, T* vpre,
+                    float* v32, unsigned vmask, bool localise, cudaStream_t s) {
+  const int n = rows.off[rows.n];
+  if (n <= 0) return;
+  // shared memory for twice the mean window, up to what leaves two blocks to an SM
+  const int cap = (int)std::min<long long>(8960, std::max<long long>(1024, 2LL * kQWin * nnz / n));
+  const size_t smem = (size_t)cap * (sizeof(double) + sizeof(int));
+  static const cudaError_t attr = cudaFuncSetAttribute(k_layouts<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                       8960 * (int)(sizeof(double) + sizeof(int)));
+  MGD_CUDA(attr);
+  k_layouts<T><<<wins.off[wins.n], kQWin, smem, s>>>(rows, wins, rp, ci, v, d, slices, sptr, sci, sv, svpre, vpre, v32,
+                                                     vmask, localise ? 1 : 0, cap);
+  MGD_LAUNCH_CHECK();
+}
+template void launch_layouts<double>(const JointOff&, const JointOff&, const JointOff&, int, const int*, int*,
+                                     const double*, const double*, const int*, int*, double*, double*, double*, float*,
+                                     unsigned, bool, cudaStream_t);
+template void launch_layouts<float>(const JointOff&, const JointOff&, const JointOff&, int, const int*, int*,
+                                    const double*, const double*, const int*, int*, float*, float*, float*, float*,
+                                    unsigned, bool, cudaStream_t);
 
 // ------------------------------------------------------------------ column scaling A D^-1
 // out = A D^-1 values (the FP64 product, rounded to T); vout, when given, the
