@@ -315,8 +315,8 @@ int mgd_fp64_issue_rate(void *stream, double *lane_ops_per_s);
  * MGD_EINVAL for a null output, MGD_ECUDA when a CUDA call fails. */
 int mgd_check_conversions(void *stream, long long *mismatches);
 
-/* Largest n accepted by mgd_relres_noalloc (its fixed work array holds n
- * doubles plus 1216 partial sums: about 4 MiB per GPU, kept until exit). */
+/* Largest n accepted by mgd_relres_noalloc (its fixed work array has room for n
+ * doubles and 1216 partial sums: about 4 MiB per GPU, kept until exit). */
 #define MGD_NOALLOC_MAX_N (1 << 19)
 
 /* True relative residual without any device allocation.  The paper has no
@@ -345,6 +345,16 @@ int mgd_check_conversions(void *stream, long long *mismatches);
  * caller.  Nothing from an earlier call is read back. */
 int mgd_relres_noalloc(int n, const int *d_rowptr, const int *d_colidx, const double *d_vals, const double *d_b,
                        const double *d_x, double *d_out, void *stream);
+
+/* As mgd_relres_noalloc for a matrix that has not been checked, whose column
+ * and value arrays hold ncol and nval entries: MGD_EINVAL, with d_out left as it
+ * is and x not read, unless rowptr[0] = 0, rowptr[n] <= ncol and nval, rowptr is
+ * non-decreasing and (with an entry at all) every one of the ncol columns is in
+ * [0, n).  The check runs on the device in front of the residual, so the call
+ * still waits once. */
+int mgd_relres_noalloc_checked(int n, int ncol, int nval, const int* d_rowptr, const int* d_colidx,
+                               const double* d_vals, const double* d_b, const double* d_x, double* d_out,
+                               void* stream);
 
 /* Kernels this library has launched in the calling process so far (a graph
  * replay counts each of its kernel nodes); a monotone counter for checking

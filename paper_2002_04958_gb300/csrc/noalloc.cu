@@ -6,8 +6,8 @@
 // after start-up, or a solver loop with a fixed, audited memory footprint.
 // The other
 // entry points of this library allocate their work space at setup; this one
-// keeps its work space (the residual vector and the partial sums of the two
-// norms) in a fixed array that lives in the library's device image instead.
+// keeps its work space (the partial sums of the two norms, and what the matrix
+// check found) in a fixed array that lives in the library's device image instead.
 //
 // The array is MGD_NOALLOC_MAX_N + 2 * kParts doubles (about 4 MiB).  Every
 // GPU that loads the library holds it until the process exits.  Calls share
@@ -36,23 +36,34 @@ static __device__ __align__(256) double g_noalloc_scratch[MGD_NOALLOC_MAX_N + 2 
 std::mutex g_mu;
 double* g_scratch_addr[kMaxDevices] = {nullptr};
 
-// r_i = b_i - sum_j a_ij x_j, stored in the scratch array
-__global__ void k_na_residual(int n, const int* __restrict__ rp, const int* __restrict__ ci,
+// What a matrix that comes unchecked may break: rowptr[0] = 0, rowptr[n] within
+// both arrays, rowptr non-decreasing, columns (if there is an entry) in [0, n)
+__global__ void k_na_check(int n, int ncol, int nval, const int* __restrict__ rp, const int* __restrict__ ci,
+                           int* __restrict__ bad) {
+  const int nnz = rp[n];
+  int wrong = rp[0] != 0 || nnz > ncol || nnz > nval;
+  const int stride = gridDim.x * blockDim.x, t0 = blockIdx.x * blockDim.x + threadIdx.x;
+  for (int i = t0; i < n; i += stride) wrong |= rp[i + 1] < rp[i];
+  if (nnz > 0)
+    for (int p = t0; p < ncol; p += stride) {
+      const int c = ci[p];
+      wrong |= c < 0 || c >= n;
+    }
+  if (__syncthreads_or(wrong) && threadIdx.x == 0) *bad = 1;
+}
+
+// r_i = b_i - sum_j a_ij x_j; part[blk] = sum of r_i^2 over this block's
+// elements, part[kParts + blk] = sum of b_i^2.  Nothing where the check failed.
+__global__ void k_na_partials(int n, const int* __restrict__ rp, const int* __restrict__ ci,
                               const double* __restrict__ v, const double* __restrict__ b,
-                              const double* __restrict__ x, double* __restrict__ r) {
+                              const double* __restrict__ x, const int* __restrict__ bad, double* __restrict__ part) {
+  if (*bad) return;
+  double sr = 0.0, sb = 0.0;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     double s = 0.0;
     for (int p = rp[i]; p < rp[i + 1]; ++p) s += v[p] * x[ci[p]];
-    r[i] = b[i] - s;
-  }
-}
-
-// part[blk] = sum of r_i^2 over this block's elements, part[kParts + blk] = sum of b_i^2
-__global__ void k_na_partials(int n, const double* __restrict__ r, const double* __restrict__ b,
-                              double* __restrict__ part) {
-  double sr = 0.0, sb = 0.0;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    sr += r[i] * r[i];
+    const double r = b[i] - s;
+    sr += r * r;
     sb += b[i] * b[i];
   }
   __shared__ double shr[kThreadsNA / 32], shb[kThreadsNA / 32];
@@ -77,7 +88,8 @@ __global__ void k_na_partials(int n, const double* __restrict__ r, const double*
 }
 
 // out[0] = ||r||, out[1] = ||b||, out[2] = ||r|| / ||b|| (0 when b = 0)
-__global__ void k_na_final(const double* __restrict__ part, double* __restrict__ out) {
+__global__ void k_na_final(const double* __restrict__ part, const int* __restrict__ bad, double* __restrict__ out) {
+  if (*bad) return;
   __shared__ double shr[kThreadsNA], shb[kThreadsNA];
   double a = 0.0, c = 0.0;
   for (int k = threadIdx.x; k < kParts; k += blockDim.x) {
@@ -124,30 +136,49 @@ int scratch_for_current_device(double** out) {
   return MGD_OK;
 }
 
-}  // namespace
-
-extern "C" int mgd_relres_noalloc(int n, const int* d_rowptr, const int* d_colidx, const double* d_vals,
-                                  const double* d_b, const double* d_x, double* d_out, void* stream) {
+// the call; with `check`, the matrix first (ncol and nval entries in its arrays)
+int relres(int n, int ncol, int nval, bool check, const int* d_rowptr, const int* d_colidx, const double* d_vals,
+           const double* d_b, const double* d_x, double* d_out, void* stream) {
   if (n < 1 || n > MGD_NOALLOC_MAX_N || !d_rowptr || !d_colidx || !d_vals || !d_b || !d_x || !d_out)
     return MGD_EINVAL;
   double* scratch = nullptr;
   int rc = scratch_for_current_device(&scratch);
   if (rc != MGD_OK) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  double* r = scratch;
-  double* part = scratch + MGD_NOALLOC_MAX_N;
-  int nb = (n + kThreadsNA - 1) / kThreadsNA;
-  if (nb > 4096) nb = 4096;
+  double* part = scratch;
+  int* bad = reinterpret_cast<int*>(scratch + 2 * kParts);
   // an error left pending by earlier, unrelated work would otherwise be
   // reported as a failure of this call's launches
   (void)cudaGetLastError();
-  k_na_residual<<<nb, kThreadsNA, 0, s>>>(n, d_rowptr, d_colidx, d_vals, d_b, d_x, r);
-  k_na_partials<<<kParts, kThreadsNA, 0, s>>>(n, r, d_b, part);
-  k_na_final<<<1, kThreadsNA, 0, s>>>(part, d_out);
+  if (cudaMemsetAsync(bad, 0, sizeof(int), s) != cudaSuccess) {
+    cudaGetLastError();
+    return MGD_ECUDA;
+  }
+  if (check) k_na_check<<<kParts, kThreadsNA, 0, s>>>(n, ncol, nval, d_rowptr, d_colidx, bad);
+  k_na_partials<<<kParts, kThreadsNA, 0, s>>>(n, d_rowptr, d_colidx, d_vals, d_b, d_x, bad, part);
+  k_na_final<<<1, kThreadsNA, 0, s>>>(part, bad, d_out);
+  int wrong = 0;
   if (cudaGetLastError() != cudaSuccess) return MGD_ECUDA;
+  if (check && cudaMemcpyAsync(&wrong, bad, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess) {
+    cudaGetLastError();
+    return MGD_ECUDA;
+  }
   if (cudaStreamSynchronize(s) != cudaSuccess) {
     cudaGetLastError();
     return MGD_ECUDA;
   }
-  return MGD_OK;
+  return wrong ? MGD_EINVAL : MGD_OK;
+}
+
+}  // namespace
+
+extern "C" int mgd_relres_noalloc(int n, const int* d_rowptr, const int* d_colidx, const double* d_vals,
+                                  const double* d_b, const double* d_x, double* d_out, void* stream) {
+  return relres(n, 0, 0, false, d_rowptr, d_colidx, d_vals, d_b, d_x, d_out, stream);
+}
+
+extern "C" int mgd_relres_noalloc_checked(int n, int ncol, int nval, const int* d_rowptr, const int* d_colidx,
+                                          const double* d_vals, const double* d_b, const double* d_x, double* d_out,
+                                          void* stream) {
+  return relres(n, ncol, nval, true, d_rowptr, d_colidx, d_vals, d_b, d_x, d_out, stream);
 }

@@ -26,7 +26,7 @@ ENTRY_POINTS = ["mgd_opts_default", "mgd_create", "mgd_setup", "mgd_update_value
                 "mgd_op_info", "mgd_level_info", "mgd_level_export", "mgd_block_vector", "mgd_coupling_dropped",
                 "mgd_profile_enable", "mgd_profile_read", "mgd_kernel_launches", "mgd_last_error", "mgd_destroy", "mgd_plan_info",
                 "mgd_setup_phases", "mgd_op_cycles", "mgd_level_keys", "mgd_precond_bench",
-                "mgd_relres_noalloc", "mgd_profile_read_fp64", "mgd_fp64_issue_rate", "mgd_setup_host",
+                "mgd_relres_noalloc", "mgd_relres_noalloc_checked", "mgd_profile_read_fp64", "mgd_fp64_issue_rate", "mgd_setup_host",
                 "mgd_check_conversions"]
 
 
@@ -94,6 +94,7 @@ def lib():
             "mgd_check_conversions": (I, [P, pLL]),
             "mgd_kernel_launches": (C.c_longlong, []),
             "mgd_relres_noalloc": (I, [I, P, P, P, P, P, P, P]),
+            "mgd_relres_noalloc_checked": (I, [I, I, I, P, P, P, P, P, P, P]),
             "mgd_setup_host": (I, [P, I, I, I, I, P, P, P, I]),
             "mgd_plan_info": (I, [P, I, I, pI, pI, pI, pI, pI, pI, pI, pI]),
             "mgd_setup_phases": (I, [P, P, I]),
@@ -131,12 +132,13 @@ def relres_noalloc(rowptr, col, val, b, x, out, stream=None):
     """||b - A x||, ||b|| and their ratio into the device tensor out[3], with no
     device allocation inside the library (see mgd_relres_noalloc).
 
-    The library reads these buffers through raw pointers without checking
-    them on the device, so everything that would make it read out of bounds
-    is checked here first: int32 rowptr (n+1) and col, float64 val, b (n),
-    x (n) and out (>= 3), all contiguous and on one CUDA device, and nnz =
-    rowptr[-1] entries in col and val.  The call runs with that device current
-    and, unless `stream` is given, on that device's current stream."""
+    The library reads these buffers through raw pointers, so everything that
+    would make it read out of bounds is checked: here, int32 rowptr (n+1) and
+    col, float64 val, b (n), x (n) and out (>= 3), all contiguous and on one
+    CUDA device; in the call, on the device, rowptr from 0 to nnz <= len(col),
+    len(val) without a decrease, and columns in [0, n).  The call runs with
+    that device current and, unless `stream` is given, on that device's current
+    stream."""
     import torch
     named = {"rowptr": rowptr, "col": col, "val": val, "b": b, "x": x, "out": out}
     for k, t in named.items():
@@ -161,16 +163,19 @@ def relres_noalloc(rowptr, col, val, b, x, out, stream=None):
     for k, t in named.items():
         if t.device != dev:
             raise ValueError(f"relres_noalloc: {k} is on {t.device}, rowptr on {dev}")
-    nnz = int(rowptr[-1].item())
-    if int(rowptr[0].item()) != 0 or nnz > col.numel() or nnz > val.numel():
-        raise ValueError(f"relres_noalloc: rowptr[0] must be 0 and rowptr[-1] = {nnz} <= len(col), len(val)")
-    if nnz > 0 and (int(col.min().item()) < 0 or int(col.max().item()) >= n
-                    or bool((rowptr[1:] < rowptr[:-1]).any().item())):
-        raise ValueError("relres_noalloc: rowptr must be non-decreasing and columns in [0, n)")
     with torch.cuda.device(dev):
-        st = stream or torch.cuda.current_stream(dev)
-        return lib().mgd_relres_noalloc(n, _ptr(rowptr), _ptr(col), _ptr(val), _ptr(b), _ptr(x), _ptr(out),
-                                        C.c_void_p(st.cuda_stream))
+        cur = torch.cuda.current_stream(dev)
+        st = stream or cur
+        if st != cur:
+            st.wait_stream(cur)
+        rc = lib().mgd_relres_noalloc_checked(n, col.numel(), val.numel(), _ptr(rowptr), _ptr(col), _ptr(val), _ptr(b),
+                                              _ptr(x), _ptr(out), C.c_void_p(st.cuda_stream))
+    if rc == 1:
+        nnz = int(rowptr[-1].item())
+        if int(rowptr[0].item()) != 0 or nnz > col.numel() or nnz > val.numel():
+            raise ValueError(f"relres_noalloc: rowptr[0] must be 0 and rowptr[-1] = {nnz} <= len(col), len(val)")
+        raise ValueError("relres_noalloc: rowptr must be non-decreasing and columns in [0, n)")
+    return rc
 
 
 def kernel_launches():

@@ -206,3 +206,33 @@ def test_joint_setup_many_operators(gpu, orc, kind, interp, prec):
     z = slv.precond_apply(torch.from_numpy(s.b)).cpu().numpy()
     zo = M.apply(s.b)
     assert np.linalg.norm(z - zo) <= (1e-12 if prec == 0 else 1e-4) * np.linalg.norm(zo)
+
+
+def test_relres_refuses_matrices_it_refused(gpu):
+    # the matrix check on the device: what the host-side checks refused, and the output stays as it was; an empty
+    # matrix may have any columns (none is read)
+    import torch
+    s = inputs.make_system(2, (31, 17), multigroup=True)
+    dev = torch.device("cuda")
+    rp, ci, va, b = (torch.from_numpy(a).to(dev) for a in (s.rowptr, s.col, s.val, s.b))
+    x = torch.zeros_like(b)
+    out = torch.full((3,), -1.0, dtype=torch.float64, device=dev)
+    assert gpu.relres_noalloc(rp, ci, va, b, x, out) == 0
+    assert out[2].item() == pytest.approx(1.0, rel=1e-14)
+
+    def changed(a, at, value):
+        a = a.clone()
+        a[at] = value
+        return a
+    bad = [(changed(rp, 0, 1), ci, va, "rowptr\\[0\\]"), (rp, ci[:-1], va, "rowptr\\[0\\]"), (rp, ci, va[:-1], "rowptr\\[0\\]"),
+           (changed(rp, 100, int(rp[101]) + 1), ci, va, "non-decreasing"), (rp, changed(ci, 500, -1), va, "columns"),
+           (rp, changed(ci, -1, s.n), va, "columns")]
+    for r, c, v, msg in bad:
+        out.fill_(-1.0)
+        with pytest.raises(ValueError, match=msg):
+            gpu.relres_noalloc(r, c.contiguous(), v.contiguous(), b, x, out)
+        assert torch.equal(out, torch.full_like(out, -1.0))
+    assert gpu.relres_noalloc(torch.zeros_like(rp), torch.full_like(ci, -7), va, b, x, out) == 0
+    assert out[0].item() == out[1].item()
+    side = torch.cuda.Stream()
+    assert gpu.relres_noalloc(rp, ci, va, b, x, out, stream=side) == 0
