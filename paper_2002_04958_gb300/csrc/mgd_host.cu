@@ -1648,6 +1648,7 @@ struct mgd_ctx {
   // FGMRES storage
   double *V = nullptr, *Z = nullptr, *w = nullptr, *r = nullptr, *hbuf = nullptr, *partial = nullptr,
          *ybuf = nullptr, *xtmp = nullptr, *btmp = nullptr;
+  cudaEvent_t h_ready = nullptr;  // the Hessenberg column of a step is on the host
   double* krylov = nullptr;  // V and Z
   size_t krylov_n = 0;
   mgd::ScratchRegion* region = nullptr;  // setup scratch of the context stream, kept like the Krylov vectors
@@ -3248,6 +3249,17 @@ static int fgmres(mgd_ctx* c, const double* b, double* x, double tol, bool trans
   auto Hm = [&](int i, int j) -> double& { return H[(size_t)i * m + j]; };
   int it = 0, status = MGD_ENOCONV;
   bool broke = false;  // an Arnoldi breakdown ended the previous cycle
+  // The host needs h before it can decide to stop, and a launch of the next
+  // step after that decision leaves the GPU idle for a copy, a wakeup and the
+  // launches (some 15 us; a step on 3,072 unknowns takes 40).  So the next
+  // step's preconditioner and product are issued behind the copy, unless the
+  // residual, at the rate of the last step, ends below the tolerance with this
+  // one; the rare step issued in vain is not counted.  Not with device-counted
+  // inverse loops, nor while kernels are being timed.
+  bool may_lead = c->prof.mask == 0;
+  for (const Step& st : c->steps)
+    if (st.loop) may_lead = false;
+  if (!c->h_ready) MGD_CUDA(cudaEventCreateWithFlags(&c->h_ready, cudaEventDisableTiming));
   for (;;) {
     int id = c->prof.begin(s, 2);
     launch_resid_f64(c->fmtMono, n, A.rp, A.ci, A.v, AS.sptr, AS.ci, AS.v, b, x, c->r, s);
@@ -3281,12 +3293,15 @@ static int fgmres(mgd_ctx* c, const double* b, double* x, double tol, bool trans
     std::fill(g.begin(), g.end(), 0.0);
     g[0] = beta;
     int j = 0;
+    bool led = false;   // step j's preconditioner and product are issued
+    double rate = 1.0;  // of the residual in the last step
     while (j < m) {
-      double* vj = c->V + (size_t)j * n;
-      double* zj = c->Z + (size_t)j * n;
-      precond_apply(c, vj, zj, trans);
+      auto apply = [&](int k) {
+        precond_apply(c, c->V + (size_t)k * n, c->Z + (size_t)k * n, trans);
+        spmv(c->Z + (size_t)k * n, c->w);
+      };
+      if (!led) apply(j);
       ++it;
-      spmv(zj, c->w);
       int nv = j + 1;
       int aid = c->prof.begin(s, 3);
       // modified Gram-Schmidt: h in hbuf[0..j], ||w||^2 in hbuf[64], v_{j+1} = w / ||w||
@@ -3306,7 +3321,10 @@ static int fgmres(mgd_ctx* c, const double* b, double* x, double tol, bool trans
       // product and the scaling
       c->prof.end(aid, 3, 8.0 * n * (c->gs.nb > 0 ? 2.0 * nv + 5.0 : 4.0 * nv + 2.0 + 2.0), s);
       MGD_CUDA(cudaMemcpyAsync(hp, c->hbuf, 65 * sizeof(double), cudaMemcpyDeviceToHost, s));
-      MGD_CUDA(cudaStreamSynchronize(s));
+      MGD_CUDA(cudaEventRecord(c->h_ready, s));
+      led = may_lead && j + 1 < m && it < c->o.max_it && std::fabs(g[j]) * rate > tol * bnorm;
+      if (led) apply(j + 1);
+      MGD_CUDA(cudaEventSynchronize(c->h_ready));
       c->prof.harvest();
       for (int i = 0; i <= j; ++i) Hm(i, j) = hp[i];
       double hn = std::sqrt(hp[64]);
@@ -3330,9 +3348,13 @@ static int fgmres(mgd_ctx* c, const double* b, double* x, double tol, bool trans
       g[j + 1] = -sn[j] * g[j];
       g[j] = cs[j] * g[j];
       c->hist.push_back(std::fabs(g[j + 1]) / bnorm);
+      rate = g[j] != 0.0 ? std::fabs(sn[j]) : 1.0;
       ++j;
       if (hn == 0.0) broke = true;
-      if (std::fabs(g[j]) <= tol * bnorm || hn == 0.0 || it >= c->o.max_it || !std::isfinite(g[j])) break;
+      if (std::fabs(g[j]) <= tol * bnorm || hn == 0.0 || it >= c->o.max_it || !std::isfinite(g[j])) {
+        if (led) (trans ? c->napplyT : c->napply)--;
+        break;
+      }
     }
     // a zero on the diagonal of the rotated Hessenberg matrix: the small
     // least-squares problem is singular, no solution in this Krylov space;
@@ -3879,6 +3901,7 @@ void mgd_destroy(mgd_ctx* c) {
   free_setup(c);
   free_krylov(c);
   free_region(c);
+  if (c->h_ready) cudaEventDestroy(c->h_ready);
   if (c->s_body) cudaStreamDestroy(c->s_body);
   for (auto cs : c->s_copy)
     if (cs) cudaStreamDestroy(cs);
