@@ -1389,13 +1389,18 @@ static int dense_level(const VBatch<T>& vb, double max_entries) {
   return vb.depth;
 }
 
-// Autotune the first fused level: time whole V-cycles with no fusion and with
-// fusion from the first level whose largest row count is below each threshold.
+// Autotune the first fused level: time whole V-cycles with every level's own
+// launches, with dense coarse levels from three first levels on, and, only where
+// no level is small enough for those, with the cluster kernel from the first
+// level whose largest row count is below each threshold (beside a dense level
+// the cluster kernel was never the fastest, and timing it took up to 60 ms).
 template <typename T>
 static void autotune_tail(Arena& ar, VBatch<T>& vb, bool keepT, bool graph, cudaStream_t s) {
   Profiler none;
   std::vector<int> cand{vb.depth};
+  const bool no_dense = dense_level(vb, kDenseMaxEntries) >= vb.depth;
   for (int thr : {4096, 16384, 65536, 262144}) {
+    if (!no_dense) break;
     int Lt = vb.depth;
     for (int l = 1; l < vb.depth; ++l) {
       auto& lp = vb.plan[l];
