@@ -373,6 +373,13 @@ struct LDesc {
     if (a_ && *a_ == 0) return; \
   } while (0)
 
+// the same with the flag's address loaded before the wait, as every descriptor
+// field should be: a load after it lengthens the chain that a small launch is
+#define MGD_SKIP_FLAG(act)             \
+  do {                                 \
+    if ((act) && *(act) == 0) return;  \
+  } while (0)
+
 // One subsystem's share of the fused coarse-level kernel: its level
 // descriptors from the first fused level to its coarsest level.
 template <typename T>

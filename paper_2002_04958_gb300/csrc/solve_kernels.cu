@@ -81,35 +81,56 @@ __device__ __forceinline__ double* resolve(const PRef& r, const IOSlots* io) {
   return io->z + r.off;
 }
 
+// The two halves of resolve: what the descriptor says, which is setup data and
+// is loaded before the dependency wait, and the current v or z, which is not.
+struct HalfRef {
+  char* p;
+  int slot;
+};
+__device__ __forceinline__ HalfRef half_ref(const PRef& r) {
+  return HalfRef{r.slot == 0 ? (char*)r.abs : (char*)nullptr + r.off * (long long)sizeof(double), r.slot};
+}
+__device__ __forceinline__ double* whole_ref(const HalfRef& h, const double* v, double* z) {
+  return (double*)(h.slot == 0 ? h.p : (h.slot == 1 ? (char*)v : (char*)z) + (h.p - (char*)nullptr));
+}
+
 // dst = (T)(a + sum_t s_t d_t (.) w_t)
 template <typename T>
 __global__ void k_produce(const ProduceDesc<T>* __restrict__ ds, int N, const IOSlots* __restrict__ io) {
-  MGD_PDL_ENTRY();
+  MGD_PDL_TRIGGER();
   const ProduceDesc<T>* d = ds + blockIdx.y;
   int k = blockIdx.x * blockDim.x + threadIdx.x;
+  const HalfRef ha = half_ref(d->a);
+  const int nt = d->nt;
+  T* const dst = d->dst;
+  MGD_PDL_WAIT();
   if (k >= N) return;
-  const double* a = resolve(d->a, io);
+  const double* a = whole_ref(ha, io->v, io->z);
   double acc = a ? a[k] : 0.0;
-  int nt = d->nt;
   for (int t = 0; t < nt; ++t) {
     const double* w = resolve(d->w[t], io);
     double term = w[k];
     if (d->d[t]) term *= d->d[t][k];
     acc += d->s[t] * term;
   }
-  d->dst[k] = from_f64<T>(acc);
+  dst[k] = from_f64<T>(acc);
 }
 
 // dst = base + s * x
 template <typename T>
 __global__ void k_consume(const ConsumeDesc<T>* __restrict__ ds, int N, const IOSlots* __restrict__ io) {
-  MGD_PDL_ENTRY();
+  MGD_PDL_TRIGGER();
   const ConsumeDesc<T>* d = ds + blockIdx.y;
   int k = blockIdx.x * blockDim.x + threadIdx.x;
+  const HalfRef hd = half_ref(d->dst), hb = half_ref(d->base);
+  const int unit = d->unit;
+  const double sc = d->s;
+  const T* const x = d->x;
+  MGD_PDL_WAIT();
   if (k >= N) return;
-  double* dst = resolve(d->dst, io);
-  const double* base = resolve(d->base, io);
-  double val = unit_times(d->unit, d->s, to_f64(d->x[k]));
+  double* dst = whole_ref(hd, io->v, io->z);
+  const double* base = whole_ref(hb, io->v, io->z);
+  double val = unit_times(unit, sc, to_f64(x[k]));
   dst[k] = base ? base[k] + val : val;
 }
 
@@ -141,13 +162,20 @@ __global__ void __launch_bounds__(kThreads) k_consume_produce(const ConsumeDesc<
   __shared__ const double* s_tw[kCpMaxTerms];
   __shared__ const double* s_td[kCpMaxTerms];
   __shared__ double s_ts[kCpMaxTerms];
-  MGD_PDL_ENTRY();
+  // the descriptors first (setup data); the current v and z after the wait
+  __shared__ unsigned char s_cbs[kCpMaxCons], s_cds[kCpMaxCons], s_pas[kCpMaxProd], s_tws[kCpMaxTerms];
+  MGD_PDL_TRIGGER();
   const int t = threadIdx.x;
+  auto half = [](const PRef& r, auto*& p, unsigned char& slot) {
+    const HalfRef h = half_ref(r);
+    p = (double*)h.p;
+    slot = (unsigned char)h.slot;
+  };
   for (int j = t; j < ncd; j += blockDim.x) {
     const ConsumeDesc<T>* d = cd + j;
     s_cx[j] = d->x;
-    s_cb[j] = resolve(d->base, io);
-    s_cdst[j] = resolve(d->dst, io);
+    half(d->base, s_cb[j], s_cbs[j]);
+    half(d->dst, s_cdst[j], s_cds[j]);
     s_cs[j] = d->s;
     s_cu[j] = d->unit;
   }
@@ -156,14 +184,27 @@ __global__ void __launch_bounds__(kThreads) k_consume_produce(const ConsumeDesc<
     int o = 0;
     for (int q = 0; q < j; ++q) o += pd[q].nt;
     s_pdst[j] = d->dst;
-    s_pa[j] = resolve(d->a, io);
+    half(d->a, s_pa[j], s_pas[j]);
     s_pt[j] = o;
     for (int u = 0; u < d->nt; ++u) {
-      s_tw[o + u] = resolve(d->w[u], io);
+      half(d->w[u], s_tw[o + u], s_tws[o + u]);
       s_td[o + u] = d->d[u];
       s_ts[o + u] = d->s[u];
     }
     if (j == npd - 1) s_pt[npd] = o + d->nt;
+  }
+  __syncthreads();
+  MGD_PDL_WAIT();
+  {
+    const double* const v = io->v;
+    double* const z = io->z;
+    auto whole = [&](auto*& p, unsigned char slot) { p = whole_ref(HalfRef{(char*)p, slot}, v, z); };
+    for (int j = t; j < ncd; j += blockDim.x) {
+      whole(s_cb[j], s_cbs[j]);
+      whole(s_cdst[j], s_cds[j]);
+    }
+    for (int j = t; j < npd; j += blockDim.x) whole(s_pa[j], s_pas[j]);
+    for (int j = t; j < s_pt[npd]; j += blockDim.x) whole(s_tw[j], s_tws[j]);
   }
   __syncthreads();
   const int k = blockIdx.x * blockDim.x + t;

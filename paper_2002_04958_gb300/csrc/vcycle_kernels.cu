@@ -29,6 +29,35 @@ constexpr int kVThreads = MGD_VTHREADS;
 #endif
 constexpr int kPre = MGD_KPRE;  // entries per lane loaded before the wait
 
+// A level's vectors, looked up in its descriptor.  A load after the dependency
+// wait lengthens the chain that a launch on a short level is, so the layouts
+// with several threads a row (short levels take those) look up before it; with
+// one thread a row the level is long, its launches overlap anyway, and the
+// registers that the addresses would hold cost more (level 0 of 21 x 884,736
+// rows: PRE 371 -> 411 us with 48 registers instead of 40).
+template <typename T, bool BEFORE>
+struct VecRefs {
+  const LDesc<T>* d;
+  T *b_ = nullptr, *x_ = nullptr, *xt_ = nullptr, *r_ = nullptr, *bc_ = nullptr;
+  const int* active_ = nullptr;
+  __device__ __forceinline__ explicit VecRefs(const LDesc<T>* desc) : d(desc) {
+    if (BEFORE) {
+      b_ = d->b;
+      x_ = d->x;
+      xt_ = d->xt;
+      r_ = d->r;
+      bc_ = d->bc;
+      active_ = d->active;
+    }
+  }
+  __device__ __forceinline__ const T* b() const { return BEFORE ? b_ : d->b; }
+  __device__ __forceinline__ T* x() const { return BEFORE ? x_ : d->x; }
+  __device__ __forceinline__ T* xt() const { return BEFORE ? xt_ : d->xt; }
+  __device__ __forceinline__ T* r() const { return BEFORE ? r_ : d->r; }
+  __device__ __forceinline__ T* bc() const { return BEFORE ? bc_ : d->bc; }
+  __device__ __forceinline__ const int* active() const { return BEFORE ? active_ : d->active; }
+};
+
 // PRE: xt = D^-1 b (zero initial guess), r = b - A xt = b - (A D^-1) b, using
 // the column-scaled copy of A so that each nonzero costs one multiply-add.
 // Levels with Q (POSTQ below) need no xt: it is not formed there.
@@ -45,15 +74,16 @@ __global__ void __launch_bounds__(kVThreads) k_pre(const LDesc<T>* __restrict__ 
   RowPre<T, kPre> R;
   row_load<T, FMT, kPre>(R, row, lane, valid, d->rp, d->ci, d->vpre, d->sptr, d->sci, d->svpre);
   T di = valid && lane == 0 ? d->dinv[row] : T(0);
+  VecRefs<T, (TPR > 1)> f(d);
   MGD_PDL_WAIT();
-  MGD_SKIP_INACTIVE(d);
-  const T* b = d->b;
+  MGD_SKIP_FLAG(f.active());
+  const T* b = f.b();
   XPlain<T> xf{b};
   T s = row_finish<T, FMT, kPre>(R, valid, d->ci, d->vpre, d->sci, d->svpre, xf);
   if (valid && lane == 0) {
     T bi = b[row];
-    if (!d->qperm) d->xt[row] = di * bi;
-    d->r[row] = bi - s;
+    if (!d->qperm) f.xt()[row] = di * bi;
+    f.r()[row] = bi - s;
   }
 }
 
@@ -71,11 +101,12 @@ __global__ void __launch_bounds__(kVThreads) k_post(const LDesc<T>* __restrict__
   RowPre<T, kPre> R;
   row_load<T, FMT, kPre>(R, row, lane, valid, d->rp, d->ci, d->v, d->sptr, d->sci, d->sv);
   T di = valid && lane == 0 ? d->dinv[row] : T(0);
+  VecRefs<T, (TPR > 1)> f(d);
   MGD_PDL_WAIT();
-  MGD_SKIP_INACTIVE(d);
-  XPlain<T> xf{d->xt};
+  MGD_SKIP_FLAG(f.active());
+  XPlain<T> xf{f.xt()};
   T s = row_finish<T, FMT, kPre>(R, valid, d->ci, d->v, d->sci, d->sv, xf);
-  if (valid && lane == 0) d->x[row] = d->xt[row] + di * (d->b[row] - s);
+  if (valid && lane == 0) f.x()[row] = f.xt()[row] + di * (f.b()[row] - s);
 }
 
 // Multi-slice forms of PRE and POST (FMT_SELL2, FMT_SELL4): each thread smooths
@@ -188,10 +219,16 @@ __global__ void __launch_bounds__(kVThreads) k_postq_csr(const LDesc<T>* __restr
   RowPre<T, kPre> R;
   row_load<T, FMT, kPre>(R, row, lane, valid, d->qrp, d->qci, d->qv, nullptr, nullptr, nullptr);
   T di = valid && lane == 0 ? d->dinv[row] : T(0);
+  const T* const xc = d->xc;
+  const T* const b = d->b;
+  const T* const r = d->r;
+  T* const x = d->x;
+  const int* const act = d->active;
   MGD_PDL_WAIT();
-  MGD_SKIP_INACTIVE(d);
-  T s = row_finish<T, FMT, kPre>(R, valid, d->qci, d->qv, nullptr, nullptr, XPlain<T>{d->xc});
-  if (valid && lane == 0) d->x[row] = di * (d->b[row] + d->r[row]) + s;
+  MGD_SKIP_FLAG(act);
+  const T br = valid && lane == 0 ? b[row] + r[row] : T(0);
+  T s = row_finish<T, FMT, kPre>(R, valid, d->qci, d->qv, nullptr, nullptr, XPlain<T>{xc});
+  if (valid && lane == 0) x[row] = di * br + s;
 }
 
 // RESTRICT: bc = R r ; PROLONG: xt += P xc  (CSR, TPR threads per row)
@@ -207,11 +244,12 @@ __global__ void __launch_bounds__(kVThreads) k_restrict(const LDesc<T>* __restri
   bool valid = row < n;
   RowPre<T, kPre> R;
   row_load<T, FMT, kPre>(R, row, lane, valid, d->rrp, d->rci, d->rv, nullptr, nullptr, nullptr);
+  VecRefs<T, (TPR > 1)> f(d);
   MGD_PDL_WAIT();
-  MGD_SKIP_INACTIVE(d);
-  XPlain<T> xf{d->r};
+  MGD_SKIP_FLAG(f.active());
+  XPlain<T> xf{f.r()};
   T s = row_finish<T, FMT, kPre>(R, valid, d->rci, d->rv, nullptr, nullptr, xf);
-  if (valid && lane == 0) d->bc[row] = s;
+  if (valid && lane == 0) f.bc()[row] = s;
 }
 
 template <typename T, int FMT>
@@ -361,9 +399,11 @@ __global__ void __launch_bounds__(kDenseThreads) k_coarse(const LDesc<T>* __rest
     for (int p = 0; p < PRE; ++p)
       pre[q][p] = i0 + q < n && lane + 32 * p < n ? __ldg(m + (size_t)q * n + lane + 32 * p) : 0.0;
   }
+  const T* const b = d->b;
+  T* const x = d->x;
+  const int* const act = d->active;
   MGD_PDL_WAIT();
-  MGD_SKIP_INACTIVE(d);
-  const T* b = d->b;
+  MGD_SKIP_FLAG(act);
 #pragma unroll
   for (int p = 0; p < PRE; ++p)
     if (lane + 32 * p < n) {
@@ -395,7 +435,7 @@ __global__ void __launch_bounds__(kDenseThreads) k_coarse(const LDesc<T>* __rest
   }
 #pragma unroll
   for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-  if ((lane & (R == 1 ? 31 : 7)) == 0 && i < n) d->x[i] = (T)t;
+  if ((lane & (R == 1 ? 31 : 7)) == 0 && i < n) x[i] = (T)t;
 }
 
 #define MGD_DISPATCH_FMT(K, fmt, maxrows, ny, s, descs)                                        \
@@ -533,13 +573,15 @@ __global__ void __launch_bounds__(kVThreads) k_gs_sweep(const LDesc<T>* __restri
   if (FMT == FMT_SELL) row_load<T, FMT, kPre>(R, q, lane, valid, nullptr, nullptr, nullptr, d->gsptr, d->gsci, d->gsv);
   else row_load<T, FMT, kPre>(R, row, lane, valid, d->rp, d->ci, d->v, nullptr, nullptr, nullptr);
   const T gd = valid && lane == 0 ? d->gdinv[row] : T(0);
-  MGD_PDL_WAIT();
-  MGD_SKIP_INACTIVE(d);
   T* const xt = d->xt;
+  const T* const b = d->b;
+  const int* const act = d->active;
+  MGD_PDL_WAIT();
+  MGD_SKIP_FLAG(act);
   XCoherent<T> xf{xt};  // xt is written by this launch's other points
   T bi = T(0), xi = T(0);
   if (valid && lane == 0) {
-    bi = d->b[row];
+    bi = b[row];
     xi = xt[row];
   }
   T s = row_finish<T, FMT, kPre>(R, valid, d->ci, d->v, d->gsci, d->gsv, xf);
@@ -559,11 +601,16 @@ __global__ void __launch_bounds__(kVThreads) k_gs_resid(const LDesc<T>* __restri
   bool valid = row < n;
   RowPre<T, kPre> R;
   row_load<T, FMT, kPre>(R, row, lane, valid, d->rp, d->ci, d->v, d->sptr, d->sci, d->sv);
+  const T* const xt = d->xt;
+  const T* const b = d->b;
+  T* const r = d->r;
+  const int* const act = d->active;
   MGD_PDL_WAIT();
-  MGD_SKIP_INACTIVE(d);
-  XPlain<T> xf{d->xt};
+  MGD_SKIP_FLAG(act);
+  const T bi = valid && lane == 0 ? b[row] : T(0);
+  XPlain<T> xf{xt};
   T s = row_finish<T, FMT, kPre>(R, valid, d->ci, d->v, d->sci, d->sv, xf);
-  if (valid && lane == 0) d->r[row] = d->b[row] - s;
+  if (valid && lane == 0) r[row] = bi - s;
 }
 
 template <typename T>
