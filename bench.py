@@ -43,8 +43,8 @@ METRIC = "FGMRES time-to-1e-8 residual (s) and V-cycle HBM GB/s, mixed/batched v
 KINDS_OF = {0: "amg", 1: "schur1", 2: "bd", 3: "schur2", 4: "amg"}
 # stored oracle solves (written by the scripts beside them, which call only the oracle)
 GOLDEN = {1: "oracle_fgmres_G1_1024x1024_schur1_exti.json", 3: "oracle_fgmres_G20_96x96x96_schur2.json"}
-ARNOLDI_KERNEL = "FGMRES orthogonalisation (k_dot_partial2, k_mgs_step2 x (j+1), k_sum_partials, k_scale_by_norm2)"
-MGS_KERNEL = "k_mgs_step2 (fused modified Gram-Schmidt step: w -= h_i v_i, partial <v_i+1, w>)"
+ARNOLDI_KERNEL = ("k_gram_schmidt (modified Gram-Schmidt of one FGMRES step and the normalisation, one cooperative "
+                  "launch)")
 
 
 def _dist():
@@ -227,7 +227,7 @@ def run_ours(args):
 
     def step(k):
         if k == 0:   # the first timed step brackets the dominant kernel classes with events
-            slv.profile(0b101001)
+            slv.profile(0b1001)
         slv.setup(sysm.G, sysm.N, rp, ci, va, args.kind)
         x, it, rr, rc = slv.solve(b, tol=args.tol)
         if args.adjoint:   # L = ||x||^2: lambda = A^-T (2x), dL/dvals = -lambda_row x_col
@@ -243,7 +243,6 @@ def run_ours(args):
             prof["l0"] = slv.profile_read(0)
             prof["l0_fp64"] = slv.profile_read_fp64(0)
             prof["arn"] = slv.profile_read(3)
-            prof["mgs"] = slv.profile_read(5)
             slv.profile(0)
         return x, it, rr
 
@@ -412,29 +411,19 @@ def run_ours(args):
                 "frac": round(a64 / rate, 4), "ops": f0,
                 "peak_source": "measured in this run (mgd_fp64_issue_rate: independent multiply-add chains, "
                                "every lane active)"}
-    level0 = {"kernel": "level-0 l1-Jacobi smoothing + residual (k_pre/k_post)",
+    level0 = {"kernel": "level-0 l1-Jacobi smoothing + residual (k_pre; k_postq or k_post)",
               "achieved": round(l0_ach, 1) if l0_ach else None, "peak": peak, "unit": "GB/s",
               "frac": round(l0_ach / peak, 4) if l0_ach else None, "launches": n0, "ms": round(t0, 4),
               "bytes_per_launch": round(by0 / max(n0, 1)), "fp64_issue": fp64,
               "traffic": _traffic_from_profiles("level0", out_workload)}
-    nm, tm, bym = prof["mgs"]
-    mgs_ach = bym / (tm * 1e-3) / 1e9 if tm > 0 else None
     arnoldi = {"kernel": ARNOLDI_KERNEL, "achieved": round(arn_ach, 1) if arn_ach else None, "peak": peak,
                "unit": "GB/s", "frac": round(arn_ach / peak, 4) if arn_ach else None, "launches": na,
                "ms": round(ta, 4), "bytes_per_launch": round(bya / max(na, 1)),
-               "note": "one launch = one orthogonalisation: first dot product, the fused steps, the norm, "
-                       "the normalisation"}
-    # class 5 brackets the j+1 step launches of each orthogonalisation together:
-    # per kernel launch, 32 n algorithmic bytes
-    nmk = int(round(bym / (32.0 * sysm.n))) if bym > 0 else 0
-    mgs = {"kernel": MGS_KERNEL, "achieved": round(mgs_ach, 1) if mgs_ach else None, "peak": peak, "unit": "GB/s",
-           "frac": round(mgs_ach / peak, 4) if mgs_ach else None, "launches": nmk, "ms": round(tm, 4),
-           "bytes_per_launch": 32 * sysm.n, "traffic": _traffic_from_profiles("mgs", out_workload),
-           "timed_as": f"{nm} bracketed groups (the steps of one orthogonalisation each)",
-           "arnoldi_class": arnoldi}
-    # the dominant kernel: the larger device time in the profiled step (the
-    # fused Gram-Schmidt step launches are timed as one class per orthogonalisation)
-    dom, other = (mgs, level0) if tm > t0 else (level0, mgs)
+               "traffic": _traffic_from_profiles("arnoldi", out_workload),
+               "note": "one launch = one orthogonalisation of n_v basis vectors: 8 n (2 n_v + 5) bytes, and one "
+                       "integer-pipe and one FP64 pass over the vectors"}
+    # the dominant kernel: the larger device time in the profiled step
+    dom, other = (arnoldi, level0) if ta > t0 else (level0, arnoldi)
     roof = {"bound": "hbm", "kernel": dom["kernel"], "achieved": dom["achieved"], "peak": peak, "unit": "GB/s",
             "frac": dom["frac"], "traffic": dom["traffic"], "peak_source": peak_kind,
             "launches": dom["launches"], "ms": dom["ms"], "bytes_per_launch": dom["bytes_per_launch"],
@@ -562,7 +551,7 @@ def _oracle_opts(args):
 
 
 def _traffic_from_profiles(name, workload):
-    """DRAM bytes per launch of kernel class `name` ("level0", "mgs") on this
+    """DRAM bytes per launch of kernel class `name` ("level0", "arnoldi") on this
     workload from the committed ncu summary, when it was taken on this workload
     from the current kernel source; else None."""
     p = os.path.join(ROOT, "profiles", "roofline_traffic.json")
@@ -580,7 +569,7 @@ def _traffic_from_profiles(name, workload):
 # kernels of the class and their launcher), else the whole file
 TRAFFIC_SOURCES = {
     "level0": (("vcycle_kernels.cu", None, None), ("row_dot.cuh", None, None)),
-    "mgs": (("solve_kernels.cu", "constexpr int kMgsU", "// v = w / ||w||: one reciprocal per block"),),
+    "arnoldi": (("arnoldi_kernels.cu", None, None),),
 }
 
 
