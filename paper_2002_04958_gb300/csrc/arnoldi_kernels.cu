@@ -1,5 +1,6 @@
 // arnoldi_kernels.cu -- one FGMRES orthogonalisation (modified Gram-Schmidt of
-// w against the basis, then the normalisation) as one cooperative grid.
+// w against the basis, then the normalisation) as one launch: a cooperative
+// grid, or one cluster where there are few unknowns.
 //
 // Modified Gram-Schmidt takes h_i = <v_i, w - sum_{k<i} h_k v_k>, one grid-wide
 // reduction after the other.  With l_ik = <v_i, v_k> the same coefficients
@@ -25,7 +26,7 @@
 // largest entry per element, of either sign.
 //
 // Measured per call with 16 vectors, against the streaming kernels: 3,072
-// unknowns 20.5 / 110.9 us, 148,074 33 / 178 us, 3.1 M 227 / 394 us, 19.5 M
+// unknowns 17.6 / 110.9 us, 148,074 33 / 178 us, 3.1 M 227 / 394 us, 19.5 M
 // 1160 / 1617 us; there the first pass takes 23 us a vector (its 156 MB at the
 // copy bandwidth) and the second 39 us, its FP64 issue slots.  The second pass
 // on the integer pipe was no faster (34 us a vector, and more per call).
@@ -87,7 +88,7 @@ __device__ __forceinline__ double unfold(const int4& f) {
 // exponent in vexp[i * nunits + u]; gram: l_ik at gram[k * 32 + i], rows < nv-1
 // given, row nv-1 written by block 0.  Writes h[0..nv-1], *nrm2 = ||w'||^2 and
 // vout = w' / ||w'|| with its exponents; w is only read.
-template <int K>
+template <int K, bool CLUSTER>
 __global__ void __launch_bounds__(kGsThreads, 1)
     k_gram_schmidt(int n, const double* __restrict__ V, long long ldv, int nv, const double* __restrict__ w,
                    int* vexp, int nunits, int share_of_short, double* gram, double* __restrict__ h,
@@ -96,7 +97,14 @@ __global__ void __launch_bounds__(kGsThreads, 1)
   __shared__ double s_gram[32 * 32];
   __shared__ double s_sum[kGsWarps][64];
   __shared__ double s_dot[64], s_h[32], s_red[kGsWarps];
-  cg::grid_group grid = cg::this_grid();
+  auto sync = [] {
+    if (CLUSTER) cg::this_cluster().sync();  // (one cluster: release and acquire of global memory within it)
+    else cg::this_grid().sync();
+  };
+  if (CLUSTER) {
+    MGD_PDL_TRIGGER();
+    MGD_PDL_WAIT();
+  }
   constexpr int U = 32 * K, H = K / 2, UI = K >= 16 ? 2 : K >= 8 ? 4 : 8;
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   // warps are numbered across the blocks, so that units spread over all SMs
@@ -185,7 +193,7 @@ __global__ void __launch_bounds__(kGsThreads, 1)
     for (int q = 0; q < kGsWarps; ++q) s += s_sum[q][t];
     part[(size_t)t * nb + blockIdx.x] = s;
   }
-  grid.sync();
+  sync();
 
   // every block: the dot products from the per-block sums (the same order in
   // all), then the triangular system, a row per lane
@@ -244,7 +252,7 @@ __global__ void __launch_bounds__(kGsThreads, 1)
     for (int q = 0; q < kGsWarps; ++q) s += s_red[q];
     part[(size_t)64 * nb + blockIdx.x] = s;
   }
-  grid.sync();
+  sync();
   double nn = 0.0;  // every warp for itself, in the same order
   for (int b = lane; b < nb; b += 32) nn += __ldcg(part + (size_t)64 * nb + b);
 #pragma unroll
@@ -284,8 +292,53 @@ __global__ void __launch_bounds__(kThreads) k_unit_exponents(int n, int unit, co
 }
 
 static const void* gs_kernel(int K) {
-  return K == 2 ? (const void*)k_gram_schmidt<2> : K == 4 ? (const void*)k_gram_schmidt<4>
-       : K == 8 ? (const void*)k_gram_schmidt<8> : (const void*)k_gram_schmidt<16>;
+  return K == 2 ? (const void*)k_gram_schmidt<2, false> : K == 4 ? (const void*)k_gram_schmidt<4, false>
+       : K == 8 ? (const void*)k_gram_schmidt<8, false> : (const void*)k_gram_schmidt<16, false>;
+}
+
+// Few unknowns: what a step takes is the launch and the two barriers, so its
+// blocks are one cluster.  Its hardware barrier takes 0.3-0.5 us where the
+// grid's takes some 2, and unlike a cooperative grid it may start on the
+// product's heels (programmatic dependent launch).  A step on 3,072 unknowns
+// 39.0 -> 35.4 us.  Sixteen SMs' FP64 pipes set the line: the kernel alone with
+// 1 / 8 / 16 / 30 vectors, grid against cluster: 3,072 unknowns 14.5 / 16.6 /
+// 20.5 / 24.8 against 12.5 / 14.6 / 17.6 / 24.8 us; 8,192 unknowns 14.5 / 18.5 /
+// 20.7 / 28.5 against 12.4 / 16.6 / 20.7 / 30.9; 24,576 unknowns 16.8 / 20.7 /
+// 24.8 / 32.8 against 16.4 / 24.8 / 35.7 / 55.5.
+constexpr int kGsClusterMax = 8192;
+
+static cudaLaunchConfig_t gs_cluster_config(int blocks, cudaLaunchAttribute (&attr)[2], cudaStream_t s) {
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = blocks;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks);
+  cfg.blockDim = dim3(kGsThreads);
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = tl_pdl ? 2 : 1;
+  return cfg;
+}
+
+// the largest cluster of the kernel that the device takes: 16 blocks (a size
+// that has to be allowed first), else the portable 8, else 0
+static int gs_cluster_blocks() {
+  for (int cs : {16, 8}) {
+    int fits = 0;
+    cudaLaunchAttribute attr[2];
+    cudaLaunchConfig_t cfg = gs_cluster_config(cs, attr, nullptr);
+    cfg.numAttrs = 1;
+    if ((cs <= 8 ||
+         cudaFuncSetAttribute(k_gram_schmidt<2, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
+             cudaSuccess) &&
+        cudaOccupancyMaxActiveClusters(&fits, k_gram_schmidt<2, true>, &cfg) == cudaSuccess && fits > 0)
+      return cs;
+    cudaGetLastError();
+  }
+  return 0;
 }
 
 GsPlan gs_plan(int n) {
@@ -298,6 +351,18 @@ GsPlan gs_plan(int n) {
   }
   if (!coop || sms <= 0 || n <= 0) return p;
   const long long lanes = (long long)sms * kGsThreads;
+  if (n <= kGsClusterMax) {
+    p.K = 2;
+    const int most = gs_cluster_blocks();
+    if (most > 0) {
+      p.nunits = cdiv(n, 32 * p.K);
+      while (p.share < 8 && p.nunits * p.share * 2 <= most * kGsWarps) p.share *= 2;
+      p.nb = 1;
+      while (p.nb < most && p.nb * kGsMinWarps < p.nunits * p.share) p.nb *= 2;
+      p.cluster = true;
+      return p;
+    }
+  }
   // long units fold less often, short ones keep every warp busy: the shortest
   // that still gives each warp one unit, then 256 entries while 512 would leave
   // a warp five or fewer (1 M unknowns, 16 vectors: 100 us against 128 us;
@@ -326,6 +391,14 @@ void launch_unit_exponents(const GsPlan& p, int n, const double* v, int* vexp, c
 void launch_gram_schmidt(const GsPlan& p, int n, const double* V, long long ldv, int nv, const double* w, int* vexp,
                          double* gram, double* h, double* nrm2, double* part, double* vout, cudaStream_t s) {
   int nunits = p.nunits, share = p.share;
+  if (p.cluster) {
+    cudaLaunchAttribute attr[2];
+    const cudaLaunchConfig_t cfg = gs_cluster_config(p.nb, attr, s);
+    MGD_CUDA(cudaLaunchKernelEx(&cfg, k_gram_schmidt<2, true>, n, V, ldv, nv, w, vexp, nunits, share, gram, h, nrm2,
+                                part, vout));
+    MGD_LAUNCH_CHECK();
+    return;
+  }
   void* args[] = {(void*)&n, (void*)&V, (void*)&ldv, (void*)&nv, (void*)&w, (void*)&vexp, (void*)&nunits,
                   (void*)&share, (void*)&gram, (void*)&h, (void*)&nrm2, (void*)&part, (void*)&vout};
   MGD_CUDA(cudaLaunchCooperativeKernel(gs_kernel(p.K), dim3(p.nb), dim3(kGsThreads), args, 0, s));

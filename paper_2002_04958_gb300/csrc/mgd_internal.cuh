@@ -676,6 +676,7 @@ void launch_scale_by_norm(int n, const double* w, const double* nrm2, double* v,
 // units of 32 K entries, nunits of them, nb blocks (0: not available)
 struct GsPlan {
   int K = 0, nunits = 0, nb = 0, share = 1;  // share: warps to a unit in the first pass
+  bool cluster = false;                      // the blocks are one cluster, not a cooperative grid
 };
 constexpr int kGsMaxUnit = 512;  // entries that may be read past the last basis vector
 GsPlan gs_plan(int n);

@@ -104,6 +104,14 @@ def test_gram_schmidt_grid_matches_streaming(gpu, dims):
         assert np.allclose(grid.history(), stream.history(), rtol=1e-4, atol=1e-13)
 
 
+# 8,190 and 8,256 unknowns, on either side of the line below which the blocks are one cluster, and clusters of one to
+# sixteen blocks (81, 1,350 and 3,072 unknowns; the smaller grids above)
+@pytest.mark.parametrize("dims", [(42, 65), (43, 64), (32, 32), (18, 25), (3, 3, 3)],
+                         ids=lambda d: "x".join(map(str, d)))
+def test_gram_schmidt_cluster_matches_streaming(gpu, dims):
+    test_gram_schmidt_grid_matches_streaming(gpu, dims)
+
+
 def test_gram_schmidt_grid_not_finite(gpu):
     # an infinity or a NaN in the right-hand side ends the solve with its status, as it did
     import torch
