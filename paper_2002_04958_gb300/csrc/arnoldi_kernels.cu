@@ -101,10 +101,9 @@ __global__ void __launch_bounds__(kGsThreads, 1)
     if (CLUSTER) cg::this_cluster().sync();  // (one cluster: release and acquire of global memory within it)
     else cg::this_grid().sync();
   };
-  if (CLUSTER) {
-    MGD_PDL_TRIGGER();
-    MGD_PDL_WAIT();
-  }
+  // (the next launch only once the ones before this are over: three deep, a
+  // kernel could start while the step's first ones still read)
+  if (CLUSTER) MGD_PDL_ENTRY();
   constexpr int U = 32 * K, H = K / 2, UI = K >= 16 ? 2 : K >= 8 ? 4 : 8;
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   // warps are numbered across the blocks, so that units spread over all SMs

@@ -81,6 +81,9 @@ __device__ __forceinline__ double* resolve(const PRef& r, const IOSlots* io) {
   return io->z + r.off;
 }
 
+// (The kernels take io without restrict: the slots change while a kernel that
+// was launched early waits, so their loads must stay behind its wait.)
+
 // The two halves of resolve: what the descriptor says, which is setup data and
 // is loaded before the dependency wait, and the current v or z, which is not.
 struct HalfRef {
@@ -96,7 +99,7 @@ __device__ __forceinline__ double* whole_ref(const HalfRef& h, const double* v, 
 
 // dst = (T)(a + sum_t s_t d_t (.) w_t)
 template <typename T>
-__global__ void k_produce(const ProduceDesc<T>* __restrict__ ds, int N, const IOSlots* __restrict__ io) {
+__global__ void k_produce(const ProduceDesc<T>* __restrict__ ds, int N, const IOSlots* io) {
   MGD_PDL_TRIGGER();
   const ProduceDesc<T>* d = ds + blockIdx.y;
   int k = blockIdx.x * blockDim.x + threadIdx.x;
@@ -118,7 +121,7 @@ __global__ void k_produce(const ProduceDesc<T>* __restrict__ ds, int N, const IO
 
 // dst = base + s * x
 template <typename T>
-__global__ void k_consume(const ConsumeDesc<T>* __restrict__ ds, int N, const IOSlots* __restrict__ io) {
+__global__ void k_consume(const ConsumeDesc<T>* __restrict__ ds, int N, const IOSlots* io) {
   MGD_PDL_TRIGGER();
   const ConsumeDesc<T>* d = ds + blockIdx.y;
   int k = blockIdx.x * blockDim.x + threadIdx.x;
@@ -150,7 +153,7 @@ constexpr int kCpGroup = 4;
 template <typename T>
 __global__ void __launch_bounds__(kThreads) k_consume_produce(const ConsumeDesc<T>* __restrict__ cd, int ncd,
                                                               const ProduceDesc<T>* __restrict__ pd, int npd, int N,
-                                                              const IOSlots* __restrict__ io) {
+                                                              const IOSlots* io) {
   __shared__ const T* s_cx[kCpMaxCons];
   __shared__ const double* s_cb[kCpMaxCons];
   __shared__ double* s_cdst[kCpMaxCons];
@@ -878,7 +881,7 @@ void launch_norm2(int n, const double* x, double* partial, double* out, cudaStre
 // PCTL step 2: r_a = v_a - A_a w_a - sum_{b != a} d_ab (.) w_b for every block a
 __global__ void k_block_resid(int N, int nc, const int* const* __restrict__ brp, const int* const* __restrict__ bci,
                               const double* const* __restrict__ bv, const double* const* __restrict__ dtab,
-                              const IOSlots* __restrict__ io, double* __restrict__ r) {
+                              const IOSlots* io, double* __restrict__ r) {
   MGD_PDL_ENTRY();
   int a = blockIdx.y;
   const double* w = io->z;  // current preconditioner output (the block-relaxed w)
