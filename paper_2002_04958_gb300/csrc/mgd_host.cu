@@ -3260,8 +3260,8 @@ static int fgmres(mgd_ctx* c, const double* b, double* x, double tol, bool trans
   int it = 0, status = MGD_ENOCONV;
   bool broke = false;  // an Arnoldi breakdown ended the previous cycle
   // The host needs h before it can decide to stop, and a launch of the next
-  // step after that decision leaves the GPU idle for a copy, a wakeup and the
-  // launches (some 15 us; a step on 3,072 unknowns takes 40).  So the next
+  // step after that decision leaves the GPU idle for a wakeup and the launches
+  // (some 10 us; a step on 3,072 unknowns takes 35).  So the next
   // step's preconditioner and product are issued behind that event, unless the
   // residual, at the rate of the last step, ends below the tolerance with this
   // one; the rare step issued in vain is not counted.  Not with device-counted
