@@ -357,7 +357,8 @@ def run_ours(args):
     if args.adjoint:
         h2d += sysm.n * 8
         d2h += sysm.nnz * 8
-    del h_rp, h_ci, h_va
+    if not args.no_e2e:
+        del h_rp, h_ci, h_va
 
     # -------------------------------------------------- variants for context (one solve each, outside the timed region)
     variants = {}
